@@ -97,6 +97,10 @@ struct CpsView {
     const int32_t *val_off;        // [n_corr + 1]: coefficients of l at values[val_off[l] ..], 4^k of them
     const int32_t *site_off;       // [M + 1]: correlators covering site k are site_ent[site_off[k] ..)
     const uint32_t *site_ent;      // (l << 16) | 4^t, t = the site's digit position in l; l ascending
+    // excitations from site r to site t: the correlators that cover one of the two, ascending, with the
+    // change of their index by an alpha electron: pair_ent[pair_off[r M + t] ..) = l << 16 | change + 32768
+    const int32_t *pair_off;       // [M * M + 1]
+    const uint32_t *pair_ent;
     const double *values;          // the coefficients (parameters), FP64, device
     const float *values32;         // FP32 copy made by the last walker (re)initialisation (mixed form)
 };

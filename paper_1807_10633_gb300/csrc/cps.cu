@@ -2,8 +2,8 @@
 //
 // Correlator l covers a few spatial sites; the Fock state of a site is n_alpha + 2 n_beta and the
 // first listed site is the least significant base-4 digit of the coefficient index.  This file
-// holds the structure object (per-site lists of the correlators covering each site, so a move's
-// ratio only visits the correlators that touch its changed orbitals, Sec. III.B), the walker state
+// holds the structure object (per-site and per-site-pair lists of the correlators covering the sites,
+// so a move's ratio only visits the correlators that touch its changed orbitals, Sec. III.B), the walker state
 // (one index per correlator), its contribution to ln|psi|, and the gradient ratio
 // d ln psi / d c_l[k] = 1/c_l[k] summed over walkers in exact 64-bit fixed point.
 // The ratio itself is evaluated inside the local-energy, CTMC and move-set kernels (eloc.cu).
@@ -239,6 +239,21 @@ vmc_status vmc_cps_create(vmc_ctx *ctx, int M, int n_corr, const int32_t *h_off,
         site_ent.insert(site_ent.end(), per_site[k].begin(), per_site[k].end());   // l ascending
         site_off[k + 1] = (int32_t)site_ent.size();
     }
+    std::vector<int32_t> pair_off((size_t)M * M + 1, 0);
+    std::vector<uint32_t> pair_ent;
+    for (int r = 0; r < M; ++r)
+        for (int s = 0; s < M; ++s) {
+            const std::vector<uint32_t> &a = per_site[r], &b = per_site[s];
+            for (size_t x = 0, y = 0; r != s && (x < a.size() || y < b.size());) {
+                const uint32_t la = x < a.size() ? a[x] >> 16 : 0xFFFFu, lb = y < b.size() ? b[y] >> 16 : 0xFFFFu;
+                const uint32_t l = la < lb ? la : lb;
+                int change = 32768;
+                if (la == l) change -= (int)(a[x++] & 0xFFFFu);
+                if (lb == l) change += (int)(b[y++] & 0xFFFFu);
+                pair_ent.push_back(l << 16 | (uint32_t)change);
+            }
+            pair_off[(size_t)r * M + s + 1] = (int32_t)pair_ent.size();
+        }
     const size_t nnz = (size_t)h_off[n_corr];
     vmc_cps *c = new vmc_cps();
     c->M = M;
@@ -250,7 +265,9 @@ vmc_status vmc_cps_create(vmc_ctx *ctx, int M, int n_corr, const int32_t *h_off,
     size_t o_soff = align256(o_val + sizeof(int32_t) * (n_corr + 1));
     size_t o_ent = align256(o_soff + sizeof(int32_t) * (M + 1));
     size_t o_v32 = align256(o_ent + sizeof(uint32_t) * (site_ent.size() + 1));
-    size_t total = align256(o_v32 + sizeof(float) * (size_t)c->n_values);
+    size_t o_poff = align256(o_v32 + sizeof(float) * (size_t)c->n_values);
+    size_t o_pent = align256(o_poff + sizeof(int32_t) * pair_off.size());
+    size_t total = align256(o_pent + sizeof(uint32_t) * (pair_ent.size() + 1));
     cudaError_t e = cudaSetDevice(ctx->device);
     if (e == cudaSuccess) e = cudaMalloc(&c->dev, total);
     char *b = (char *)c->dev;
@@ -260,6 +277,9 @@ vmc_status vmc_cps_create(vmc_ctx *ctx, int M, int n_corr, const int32_t *h_off,
     if (e == cudaSuccess) e = cudaMemcpy(b + o_soff, site_off.data(), sizeof(int32_t) * (M + 1), cudaMemcpyHostToDevice);
     if (e == cudaSuccess && !site_ent.empty())
         e = cudaMemcpy(b + o_ent, site_ent.data(), sizeof(uint32_t) * site_ent.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(b + o_poff, pair_off.data(), sizeof(int32_t) * pair_off.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && !pair_ent.empty())
+        e = cudaMemcpy(b + o_pent, pair_ent.data(), sizeof(uint32_t) * pair_ent.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         vmc_cps_destroy(c);
         return cuda_check(ctx, e, "correlator structure upload");
@@ -274,6 +294,8 @@ vmc_status vmc_cps_create(vmc_ctx *ctx, int M, int n_corr, const int32_t *h_off,
     v.values32 = (const float *)(b + o_v32);
     v.site_off = (const int32_t *)(b + o_soff);
     v.site_ent = (const uint32_t *)(b + o_ent);
+    v.pair_off = (const int32_t *)(b + o_poff);
+    v.pair_ent = (const uint32_t *)(b + o_pent);
     v.values = nullptr;
     *out = c;
     return VMC_OK;
