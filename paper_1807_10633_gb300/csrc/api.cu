@@ -35,25 +35,6 @@ vmc_status ensure_workspace(vmc_ctx *ctx, size_t bytes) {
     return VMC_OK;
 }
 
-static vmc_status ensure_rates(vmc_ctx *ctx, size_t bytes, void **out) {
-    static_assert(sizeof(u128) == 16, "u128");
-    // the rate store has its own allocation: it must survive the gradient's use of ctx->ws
-    if (bytes > ctx->rates_bytes) {
-        if (ctx->rates) {
-            cudaError_t e = cudaStreamSynchronize(ctx->stream);
-            if (e != cudaSuccess) return cuda_check(ctx, e, "rate store resize");
-            cudaFree(ctx->rates);
-            ctx->rates = nullptr;
-            ctx->rates_bytes = 0;
-        }
-        cudaError_t e = cudaMalloc(&ctx->rates, bytes);
-        if (e != cudaSuccess) return cuda_check(ctx, e, "rate store");
-        ctx->rates_bytes = bytes;
-    }
-    *out = ctx->rates;
-    return VMC_OK;
-}
-
 size_t walker_stride_G(int M, int na, int nb) { return (size_t)(M - na) * na + (size_t)(M - nb) * nb; }
 size_t walker_stride_A(int na, int nb) { return (size_t)na * na + (size_t)nb * nb; }
 
@@ -206,10 +187,7 @@ vmc_status vmc_local_energy(vmc_ctx *ctx, const vmc_lists *Lc, const vmc_params 
     st = lists_set_eps(ctx, L, eps_run);
     if (st) return st;
     const int ng = L->view.n_groups;
-    void *rates = nullptr;
-    st = ensure_rates(ctx, sizeof(u128) * rate_store_units(Wk->W, ng), &rates);
-    if (st) return st;
-    st = launch_local_energy(ctx, L, Wk, cps_view(P), e_loc, t_res, (u128 *)rates, ng);
+    st = launch_local_energy(ctx, L, Wk, cps_view(P), e_loc, t_res);
     if (st) return st;
     ctx->rates_walkers = Wk->G;
     ctx->rates_groups = ng;

@@ -28,8 +28,12 @@ struct vmc_ctx {
     std::string err;
     void *ws = nullptr;          // scratch for gradient partial sums
     size_t ws_bytes = 0;
-    void *rates = nullptr;       // CTMC rate store: per walker, per group, 128-bit sums
+    // CTMC rate store (per walker, per group, 128-bit sums), then free-entry rows: its own allocation, which
+    // survives the gradient's use of ws
+    void *rates = nullptr;
     size_t rates_bytes = 0;
+    void *bits = nullptr;        // in rates: the free-entry rows of the last vmc_local_energy's walkers
+    int bits_whole = 0;          // they hold every walker of the last vmc_local_energy
     // rate store bookkeeping (vmc_local_energy -> vmc_ctmc_step)
     const void *rates_walkers = nullptr;
     int rates_valid = 0;
@@ -58,21 +62,27 @@ struct ListsView {
     int n_groups;  // singles blocks of 32 spin orbitals + M * cpr alpha-row chunks + beta groups
     int64_t ns, nds, ndo;
     int64_t ns_pad;          // ns rounded up to a multiple of 4: row stride of the Fock tables and of F
-    // singles, CSR over spatial i; records {a, w_alpha, w_beta, 0}: 16 B (mixed) or 32 B (FP64,
-    // the first 8 bytes hold a)
-    const uint32_t *s_off, *s_len, *s_owner;
+    // singles: owner i and target a of entry e (the Fock tables and F are indexed by it)
+    const uint32_t *s_owner;
     const uint16_t *s_a;
-    const float4 *s_rec32;
-    const double4_32a *s_rec64;
-    // same-spin doubles, CSR over tri(p<q); records: mixed {ab, v, w_alpha, w_beta},
-    // FP64 {ab, v, w_alpha, w_beta} with ab in the first 8 bytes
-    const uint32_t *ds_off, *ds_len, *ds_ab, *ds_owner;
-    const float4 *ds_rec32;
-    const double4_32a *ds_rec64;
-    // opposite-spin doubles, CSR over p*M+q; records {ab, v, w, 0}
-    const uint32_t *do_off, *do_len, *do_ab, *do_owner;
-    const float4 *do_rec32;
-    const double4_32a *do_rec64;
+    // every move of the walk in canonical order ("flat" entries): the lists of a group's units one
+    // after the other; each group starts on an even word of 32 entries, its opposite-spin part and a
+    // change of spin among singles on a word (unused places: key 0, never alive).  Same-spin lists
+    // and singles stand there once per spin.
+    //   key   a | b << 8 | i << 16 | j << 24, spatial orbitals (singles: b = a, j = i)
+    //   wcls  per word: bit 0 = spin of a and i, bit 1 = spin of b and j
+    //   alive per word: the entries above the current eps_run
+    //   rec   {key, v, w, aux}: integral, Jastrow constant; aux = index into a walker's F (singles)
+    //   group {first word, first opposite-spin word, end word, units}: units bit 0 = spin of the same-spin
+    //         part; the unit of an entry stands in lane (modulo 32) j + i ui + u0 (same spin; ui = bits
+    //         1-5, u0 = bits 6-10), j + u2 (opposite spin; u2 = bits 11-15), spin orbital i (singles)
+    int words;               // flat words, a multiple of 8
+    int scaled;              // FP64 local energy: G scaled by E_a / E_i once per walker (else per entry)
+    const uint32_t *key, *alive;
+    const uint8_t *wcls;
+    const float4 *rec32;
+    const double4_32a *rec64;
+    const uint4 *group;
     // Fock-sum update tables: Tj[k][e] = (ai|kk), Tjk[k][e] = (ai|kk) - (ak|ki), rows of ns_pad
     // (zero padded); FP64 and FP32 copies
     const double *Tj, *Tjk;
@@ -81,7 +91,7 @@ struct ListsView {
     const double *Jd, *Kd, *hd, *h1;
     double e_core;
     // work units of the local energy, [n_groups][32] in canonical order: {key naming the unit's own
-    // orbitals (a | b << 16, spatial for kinds 0-1, alpha | beta << 16 for kind 2), list base,
+    // orbitals (a | b << 16, spatial for kinds 0-1, alpha | beta << 16 for kind 2), flat base,
     // list length at the current eps_run (0: no unit), kind | spin << 2}
     const uint4 *unit_tab;
 };
@@ -121,6 +131,7 @@ struct vmc_lists {
     // host copies of the sorted magnitudes (for effective lengths at a given eps_run)
     double *h_s_key = nullptr, *h_ds_key = nullptr, *h_do_key = nullptr;
     uint32_t *h_s_off = nullptr, *h_ds_off = nullptr, *h_do_off = nullptr;
+    uint32_t *h_base = nullptr;   // flat base of every unit, [n_groups][32]
     void *dev = nullptr;     // one device allocation holding every array
     size_t dev_bytes = 0;
     ListsView view{};
@@ -223,6 +234,29 @@ __device__ __forceinline__ uint64_t philox4x64_word0(uint64_t c0, uint64_t c1, u
     return c0;
 }
 
+// Dependent launches: a kernel launched by launch_dependent may start while the kernel before it on the
+// stream still runs, once all CTAs of that one have called launch_dependents (or ended); what the earlier
+// kernel writes may be read only after wait_dependency (which returns at once in an ordinary launch).  So
+// `dependent` is set only where the kernel before is one of this library's, itself launched ordinarily, and
+// the kernel waits before it touches that one's output.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_dependency() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... KArgs, typename... Args>
+cudaError_t launch_dependent(bool dependent, void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t stream, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute a = {};
+    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a.val.programmaticStreamSerializationAllowed = dependent ? 1 : 0;
+    cfg.attrs = &a;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
 // ------------------------------------------------------------------ host-side helpers
 vmc_status set_err(vmc_ctx *ctx, vmc_status st, const std::string &msg);
 vmc_status cuda_check(vmc_ctx *ctx, cudaError_t e, const char *what);
@@ -236,7 +270,7 @@ vmc_status launch_init_walkers(vmc_ctx *ctx, vmc_lists *L, const vmc_params *P,
                                vmc_walkers *Wk, int full);
 struct CpsView;
 vmc_status launch_local_energy(vmc_ctx *ctx, const vmc_lists *L, vmc_walkers *Wk, const CpsView &C,
-                               double *e_loc, double *t_res, u128 *rates, int n_groups);
+                               double *e_loc, double *t_res);
 vmc_status launch_ctmc_step(vmc_ctx *ctx, const vmc_lists *L, const vmc_params *P,
                             vmc_walkers *Wk, uint64_t seed, const u128 *rates, int n_groups,
                             uint64_t *move_code);

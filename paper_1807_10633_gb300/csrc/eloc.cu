@@ -18,6 +18,7 @@
 
 #include <algorithm>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -26,12 +27,18 @@ namespace {
 
 __device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ float rmul(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double rsub(double a, double b) { return __dsub_rn(a, b); }
 __device__ __forceinline__ float rsub(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ double rexp(double x) { return exp(x); }
 __device__ __forceinline__ float rexp(float x) { return expf(x); }
 __device__ __forceinline__ double rrcp(double x) { return __ddiv_rn(1.0, x); }
 __device__ __forceinline__ float rrcp(float x) { return __fdiv_rn(1.0f, x); }
+
+__device__ __forceinline__ unsigned long long abs_bits(double v) {
+    return (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
+}
+// 2 x 2 minor of G; accumulation of a contribution (FP64 form: fused, the FP64 pipe is its bound)
+__device__ __forceinline__ float minor2(float a, float d, float b, float c) { return rsub(rmul(a, d), rmul(b, c)); }
+__device__ __forceinline__ double minor2(double a, double d, double b, double c) { return __fma_rn(a, d, -__dmul_rn(b, c)); }
 
 // 16-byte vectors of the table precision, and f += sgn * x on them
 template <typename real> struct Vec16;
@@ -59,29 +66,11 @@ template <> __device__ __forceinline__ const double *fock_table<double>(const Li
     return same ? L.Tjk : L.Tj;
 }
 
-// One packed list record (16 B in the mixed form, 32 B in the FP64 form): key (a or a|b<<16)
-// and up to three reals.
-template <typename real> struct Rec;
-template <> struct Rec<float> {
-    float4 v;
-    __device__ uint32_t key() const { return __float_as_uint(v.x); }
-    __device__ float f1() const { return v.y; }
-    __device__ float f2() const { return v.z; }
-    __device__ float f3() const { return v.w; }
-};
-template <> struct Rec<double> {
-    double4_32a v;
-    __device__ uint32_t key() const { return (uint32_t)__double_as_longlong(v.x); }
-    __device__ double f1() const { return v.y; }
-    __device__ double f2() const { return v.z; }
-    __device__ double f3() const { return v.w; }
-};
-__device__ __forceinline__ Rec<float> rec_single(const ListsView &L, uint32_t e, float) { return Rec<float>{__ldg(&L.s_rec32[e])}; }
-__device__ __forceinline__ Rec<double> rec_single(const ListsView &L, uint32_t e, double) { return Rec<double>{L.s_rec64[e]}; }
-__device__ __forceinline__ Rec<float> rec_same(const ListsView &L, uint32_t e, float) { return Rec<float>{__ldg(&L.ds_rec32[e])}; }
-__device__ __forceinline__ Rec<double> rec_same(const ListsView &L, uint32_t e, double) { return Rec<double>{L.ds_rec64[e]}; }
-__device__ __forceinline__ Rec<float> rec_opp(const ListsView &L, uint32_t e, float) { return Rec<float>{__ldg(&L.do_rec32[e])}; }
-__device__ __forceinline__ Rec<double> rec_opp(const ListsView &L, uint32_t e, double) { return Rec<double>{L.do_rec64[e]}; }
+// Record of a flat entry: {key, integral, Jastrow constant, index into F}.
+__device__ __forceinline__ float4 flat_rec(const ListsView &L, uint32_t e, float) { return __ldg(&L.rec32[e]); }
+__device__ __forceinline__ double4_32a flat_rec(const ListsView &L, uint32_t e, double) { return L.rec64[e]; }
+__device__ __forceinline__ uint32_t low_bits(float x) { return __float_as_uint(x); }
+__device__ __forceinline__ uint32_t low_bits(double x) { return (uint32_t)__double_as_longlong(x); }
 
 // Walker arrays (global) and geometry.
 struct WalkerArgs {
@@ -102,7 +91,9 @@ struct SysDesc {
     double *e_loc, *t_res;
     u128 *rates;
     uint64_t *move_code;
-    int w_begin;
+    uint32_t *bits;          // free-entry rows of walkers w_first .. w_first + w_count - 1
+    int w_first, w_count;    // the walkers of this launch (a batch may take several rounds)
+    int w_begin, t_begin;    // first position of the system in the launch: walkers, walker tiles
 };
 
 struct Geo {
@@ -125,13 +116,13 @@ __device__ __forceinline__ Geo make_geo(int M, int na, int nb) {
 // A work unit: one occupied spin orbital (single) or one occupied pair (double).
 template <typename real>
 struct Unit {
-    uint32_t base, len;
+    uint32_t base, len;   // flat entries
     int kind;      // 0 single, 1 same-spin double, 2 opposite-spin double
     int cls;       // spin for kinds 0 and 1
     int ci, cj;    // columns of i and j
     int i, j;      // spin orbitals
     uint32_t sent; // key naming the unit's own (occupied) orbitals
-    real einv;     // (1/E_i)(1/E_j)   (1/E_i for singles)
+    real ei, ej;   // 1/E_i, 1/E_j
 };
 
 // Shared-memory view of one walker used by the entry evaluation.
@@ -223,19 +214,19 @@ __device__ __forceinline__ bool setup_unit(const ListsView &L, const View<real> 
     const int M = L.M;
     const uint4 t = __ldg(&L.unit_tab[(size_t)g * 32 + lane]);
     u.base = t.y; u.len = t.z; u.kind = (int)(t.w & 3); u.cls = (int)(t.w >> 2); u.sent = t.x;
-    u.ci = 0; u.cj = 0; u.einv = real(0);
+    u.ci = 0; u.cj = 0; u.ei = u.ej = real(0);
     const int lo = (int)(t.x & 0xFFFFu), hi = (int)(t.x >> 16);
     u.i = u.kind == 2 ? lo : u.cls * M + lo;
     u.j = u.kind == 0 ? -1 : (u.kind == 2 ? M + hi : u.cls * M + hi);
-    if (u.len == 0 || !V.occ(u.i)) return false;
-    if (u.kind != 0 && !V.occ(u.j)) return false;
+    if (u.len == 0) return false;
     u.ci = V.pos[u.i];
-    if (u.kind == 0) {
-        u.einv = V.Eiv(u.i);
-    } else {
+    if (u.ci & 0x8000) return false;
+    if (u.kind != 0) {
         u.cj = V.pos[u.j];
-        u.einv = rmul(V.Eiv(u.i), V.Eiv(u.j));
+        if (u.cj & 0x8000) return false;
+        u.ej = V.Eiv(u.j);
     }
+    u.ei = V.Eiv(u.i);
     return true;
 }
 
@@ -250,26 +241,17 @@ __device__ __forceinline__ Unit<real> shfl_unit(const Unit<real> &u, int src) {
     v.cj = __shfl_sync(0xffffffffu, u.cj, src);
     v.i = __shfl_sync(0xffffffffu, u.i, src);
     v.j = __shfl_sync(0xffffffffu, u.j, src);
-    v.einv = __shfl_sync(0xffffffffu, u.einv, src);
+    v.ei = __shfl_sync(0xffffffffu, u.ei, src);
+    v.ej = __shfl_sync(0xffffffffu, u.ej, src);
     return v;
 }
 
-// Are the target orbital(s) of entry idx unoccupied?  Reads only the 2- or 4-byte key.
+// Are the target orbital(s) of flat entry e unoccupied?
 template <typename real>
-__device__ __forceinline__ bool entry_free(const ListsView &L, const View<real> &V, int kind, int cls,
-                                           uint32_t idx) {
-    const int M = V.geo.M;
-    if (kind == 0) return V.pos[cls * M + __ldg(&L.s_a[idx])] & 0x8000;
-    if (kind == 1) {
-        const uint32_t ab = __ldg(&L.ds_ab[idx]);
-        return V.pos[cls * M + (ab & 0xFFFF)] & V.pos[cls * M + (ab >> 16)] & 0x8000;
-    }
-    const uint32_t ab = __ldg(&L.do_ab[idx]);
-    return V.pos[ab & 0xFFFF] & V.pos[M + (ab >> 16)] & 0x8000;
-}
-
-__device__ __forceinline__ uint32_t list_size(const ListsView &L, int kind) {
-    return (uint32_t)(kind == 0 ? L.ns : (kind == 1 ? L.nds : L.ndo));
+__device__ __forceinline__ bool entry_free(const ListsView &L, const View<real> &V, int kind, int cls, uint32_t e) {
+    const int M = V.geo.M, sa = kind == 2 ? 0 : cls * M, sb = kind == 2 ? M : sa;
+    const uint32_t key = __ldg(&L.key[e]);
+    return V.pos[sa + (key & 0xFFu)] & V.pos[sb + (key >> 8 & 0xFFu)] & 0x8000;
 }
 
 // ratio = psi(m)/psi(n) of a free entry (in-place replacement convention: the fermionic phases
@@ -277,48 +259,57 @@ __device__ __forceinline__ uint32_t list_size(const ListsView &L, int kind) {
 // this one sequence of explicitly rounded operations, so they agree bit for bit.
 template <typename real, bool kC>
 __device__ __forceinline__ void entry_value(const ListsView &L, const View<real> &V, int kind, int cls, int ci,
-                                            int cj, real einv, uint32_t idx, real &ratio, real &contrib, int &A,
+                                            int cj, real ei, real ej, uint32_t e, real &ratio, real &contrib, int &A,
                                             int &B, int I = -1, int Jo = -1) {
     const int M = V.geo.M;
+    const auto r = flat_rec(L, e, real(0));
+    const uint32_t key = low_bits(r.x);
+    const int s = cls, a = (int)(key & 0xFFu), b = (int)(key >> 8 & 0xFFu);
+    // FP64 form with long lists: G elements scaled by E_a / E_i first; otherwise the factors one after the other
+    const bool scaled = sizeof(real) == 8 && L.scaled;
+    auto elem = [&](int sp, int k, int c, real eic) {
+        const real g = V.Grow(sp, V.pos[sp * M + k] & 0x7FFF)[c];
+        return scaled ? rmul(rmul(g, V.Ev(sp * M + k)), eic) : g;
+    };
     if (kind == 0) {
-        const int s = cls;
-        const Rec<real> r = rec_single(L, idx, real(0));
-        const int a = (int)r.key();
-        const real g = V.Grow(s, V.pos[s * M + a] & 0x7FFF)[ci];
-        const real w = s ? r.f2() : r.f1();
-        real rt = rmul(rmul(rmul(g, w), V.Ev(s * M + a)), einv);
+        const real g = elem(s, a, ci, ei);
+        real rt = scaled ? rmul(g, r.z) : rmul(rmul(rmul(g, r.z), V.Ev(s * M + a)), ei);
         if (kC) rt = rmul(rt, cps_ratio<real>(V, I, s * M + a, I, s * M + a, 2));
         ratio = rt;
-        contrib = rmul(V.F[(size_t)s * L.ns_pad + idx], rt);
+        contrib = rmul(V.F[low_bits(r.w)], rt);
         A = s * M + a; B = -1;
         return;
     }
+    real x;
     if (kind == 1) {
-        const int s = cls;
-        const Rec<real> r = rec_same(L, idx, real(0));
-        const uint32_t ab = r.key();
-        const int a = ab & 0xFFFF, b = ab >> 16;
-        const real *ra = V.Grow(s, V.pos[s * M + a] & 0x7FFF);
-        const real *rb = V.Grow(s, V.pos[s * M + b] & 0x7FFF);
-        const real minor = rsub(rmul(ra[ci], rb[cj]), rmul(ra[cj], rb[ci]));
-        const real w = s ? r.f3() : r.f2();
-        real rt = rmul(rmul(rmul(rmul(minor, w), V.Ev(s * M + a)), V.Ev(s * M + b)), einv);
-        if (kC) rt = rmul(rt, cps_ratio<real>(V, I, s * M + a, Jo, s * M + b, 4));
-        ratio = rt;
-        contrib = rmul(r.f1(), rt);
+        x = minor2(elem(s, a, ci, ei), elem(s, b, cj, ej), elem(s, a, cj, ej), elem(s, b, ci, ei));
         A = s * M + a; B = s * M + b;
-        return;
+    } else {
+        x = rmul(elem(0, a, ci, ei), elem(1, b, cj, ej));
+        A = a; B = M + b;
     }
-    const Rec<real> r = rec_opp(L, idx, real(0));
-    const uint32_t ab = r.key();
-    const int a = ab & 0xFFFF, b = ab >> 16;
-    const real ga = V.Grow(0, V.pos[a] & 0x7FFF)[ci];
-    const real gb = V.Grow(1, V.pos[M + b] & 0x7FFF)[cj];
-    real rt = rmul(rmul(rmul(rmul(rmul(ga, gb), r.f2()), V.Ev(a)), V.Ev(M + b)), einv);
-    if (kC) rt = rmul(rt, cps_ratio<real>(V, I, a, Jo, M + b, 4));
+    real rt = rmul(x, r.z);
+    if (!scaled) rt = rmul(rmul(rmul(rt, V.Ev(A)), V.Ev(B)), rmul(ei, ej));
+    if (kC) rt = rmul(rt, cps_ratio<real>(V, I, A, Jo, B, 4));
     ratio = rt;
-    contrib = rmul(r.f1(), rt);
-    A = a; B = M + b;
+    contrib = rmul(r.y, rt);
+}
+
+// The same for flat entry e of any unit (its orbitals from the key): ratio, contribution and move code.
+// False if it is no move of this walker (bits of other walkers or occupations: nothing is read then).
+template <typename real, bool kC>
+__device__ __forceinline__ bool flat_entry_value(const ListsView &L, const View<real> &V, bool single, uint32_t e,
+                                                 real &ratio, real &contrib, uint64_t &code) {
+    const int M = V.geo.M, cls = __ldg(&L.wcls[e >> 5]), sa = cls & 1, sb = cls >> 1;
+    const uint32_t key = __ldg(&L.key[e]);
+    const int I = sa * M + (int)(key >> 16 & 0xFFu), J = sb * M + (int)(key >> 24);
+    int A = sa * M + (int)(key & 0xFFu), B = sb * M + (int)(key >> 8 & 0xFFu);
+    if ((V.pos[I] | V.pos[J] | ~(V.pos[A] & V.pos[B])) & 0x8000) return false;
+    entry_value<real, kC>(L, V, single ? 0 : (sa == sb ? 1 : 2), sa, V.pos[I], V.pos[J], V.Eiv(I),
+                          single ? real(0) : V.Eiv(J), e, ratio, contrib, A, B, I, J);
+    code = single ? 1ull | (uint64_t)I << 2 | 1023ull << 12 | (uint64_t)A << 22 | 1023ull << 32
+                  : 2ull | (uint64_t)I << 2 | (uint64_t)J << 12 | (uint64_t)A << 22 | (uint64_t)B << 32;
+    return true;
 }
 
 // Evaluate list entry `idx` of unit u.  Returns false if the target orbital(s) are occupied.
@@ -326,7 +317,7 @@ template <typename real, bool kC>
 __device__ __forceinline__ bool eval_entry(const ListsView &L, const View<real> &V, const Unit<real> &u,
                                            uint32_t idx, real &ratio, real &contrib, int &A, int &B) {
     if (!entry_free<real>(L, V, u.kind, u.cls, idx)) return false;
-    entry_value<real, kC>(L, V, u.kind, u.cls, u.ci, u.cj, u.einv, idx, ratio, contrib, A, B, u.i, u.j);
+    entry_value<real, kC>(L, V, u.kind, u.cls, u.ci, u.cj, u.ei, u.ej, idx, ratio, contrib, A, B, u.i, u.j);
     return true;
 }
 
@@ -350,139 +341,393 @@ __device__ __forceinline__ double warp_sum_acc(float v) {
     return (double)v;
 }
 
-// Evaluate cnt queued entries q[0..cnt) of one warp, one per lane (lanes >= cnt idle).  Every entry
-// of one queue has the same kind K (compile time).  Entry code = list index << 5 | unit lane; the
-// unit's columns, 1/(E_i E_j) and kind | spin << 2 are held by that lane (cci, ccj, ceinv, cmeta).
-template <int K, typename real, typename acc_t, bool kC>
-__device__ __forceinline__ void drain_queue(const ListsView &L, const View<real> &V, const uint32_t *q, int cnt,
-                                            int lane, int cci, int ccj, real ceinv, int cmeta, int cii, int cjj,
-                                            acc_t &e_grp, u128 &q_grp, unsigned &flag) {
-    const uint32_t code = lane < cnt ? q[lane] : 0u;
-    const int src = (int)(code & 31u);
-    const int ci = __shfl_sync(0xffffffffu, cci, src);
-    const int cj = K == 0 ? 0 : __shfl_sync(0xffffffffu, ccj, src);
-    const real einv = __shfl_sync(0xffffffffu, ceinv, src);
-    const int cls = K == 2 ? 0 : (__shfl_sync(0xffffffffu, cmeta, src) >> 2);
-    const int oi = kC ? __shfl_sync(0xffffffffu, cii, src) : -1;
-    const int oj = (kC && K != 0) ? __shfl_sync(0xffffffffu, cjj, src) : -1;
-    if (lane < cnt) {
-        real ratio, contrib;
-        int a, b;
-        entry_value<real, kC>(L, V, K, cls, ci, cj, einv, code >> 5, ratio, contrib, a, b, oi, oj);
-        e_grp += (acc_t)contrib;
-        q_grp += rate_of<real>(ratio, &flag);
+// ---------------------------------------------------------------------------------- free entries
+// 32 x 32 bit transpose across a warp: lane l holds row l; afterwards lane l holds column l.
+__device__ __forceinline__ uint32_t transpose_bits(uint32_t x, int lane) {
+#pragma unroll
+    for (int k = 16; k >= 1; k >>= 1) {
+        const uint32_t m = k == 16 ? 0x0000FFFFu : k == 8 ? 0x00FF00FFu : k == 4 ? 0x0F0F0F0Fu : k == 2 ? 0x33333333u : 0x55555555u;
+        const uint32_t y = __shfl_xor_sync(0xffffffffu, x, k);
+        const uint32_t keep = (lane & k) ? ~m : m;
+        const uint32_t r = __funnelshift_l(y, y, (lane & k) ? 32 - k : k);
+        x = (x & keep) | (r & ~keep);
+    }
+    return x;
+}
+
+// Which flat entries are moves, for tiles of 64 walkers: one bit per entry and walker, set if i and j
+// are occupied, a and b empty and the entry is above eps_run.  A warp takes 256 consecutive entries:
+// lane = entry, the 64 walkers' occupations of an orbital are two words (bit = walker) in shared
+// memory, so a few logic operations answer 64 walkers; bit transposes turn lane = entry into
+// lane = walker, and every walker's 32 bytes are stored as one sector.
+// Grid: (tiles of 64 walkers, splits of the row).  The local energy is launched as its dependent: it stages its
+// tables meanwhile and waits before it reads the first bits.
+constexpr int kTile = 64;
+
+// Rows of at most this many words are made by the local energy's own CTA (a warp per word, lane = entry):
+// at 10 orbitals that is one launch less; from a few hundred words on the tiles of walkers win.
+constexpr int kOwnWords = 64;
+// While all CTAs are resident at once (four per SM) the launch counts for more: 300 walkers of H14 at
+// eps = 1e-4 (about 100 words) 12.5 -> 12.0 us.
+constexpr int kOwnWordsSmall = 256, kOwnWalkers = 608;
+inline bool own_rows(int words, int W) { return words <= kOwnWords || (words <= kOwnWordsSmall && W <= kOwnWalkers); }
+
+__device__ __forceinline__ void free_bits_tile(const ListsView &L, const uint32_t *__restrict__ occ_bits, int w_first,
+                                               int w_end, int tile, int part, int parts, uint32_t *__restrict__ bits,
+                                               uint2 *s_occ) {
+    const int M = L.M, nw = (M + 31) / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+    const int w = w_first + tile * kTile + lane;     // this lane's walkers: w and w + 32
+    // s_occ[p]: bit l set if spin orbital p is occupied in walker l of the tile
+    for (int t = warp; t < 2 * nw; t += nwarp) {
+        const int s = t / nw, k0 = (t - s * nw) * 32;
+        const uint32_t x = transpose_bits(w < w_end ? occ_bits[(size_t)w * 2 * nw + t] : 0u, lane);
+        const uint32_t y = transpose_bits(w + 32 < w_end ? occ_bits[(size_t)(w + 32) * 2 * nw + t] : 0u, lane);
+        if (k0 + lane < M) s_occ[s * M + k0 + lane] = make_uint2(x, y);
+    }
+    __syncthreads();
+    uint32_t *row = bits + (size_t)(tile * kTile + lane) * L.words;
+    for (int c = part * nwarp + warp; c * 8 < L.words; c += parts * nwarp) {
+        uint32_t key[8], x[8], y[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) key[j] = __ldg(&L.key[c * 256 + 32 * j + lane]);
+        const uint2 cl = __ldg((const uint2 *)(L.wcls + c * 8));
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const uint32_t cls = (j < 4 ? cl.x : cl.y) >> (8 * (j & 3));
+            const uint2 *oa = s_occ + ((cls & 1u) ? M : 0), *ob = s_occ + ((cls & 2u) ? M : 0);
+            const uint32_t k = key[j];
+            const uint2 a = oa[k & 0xFFu], b = ob[k >> 8 & 0xFFu], i = oa[k >> 16 & 0xFFu], q = ob[k >> 24];
+            x[j] = transpose_bits(i.x & q.x & ~(a.x | b.x), lane);
+            y[j] = transpose_bits(i.y & q.y & ~(a.y | b.y), lane);
+        }
+        const uint4 l0 = __ldg((const uint4 *)(L.alive + c * 8)), l1 = __ldg((const uint4 *)(L.alive + c * 8 + 4));
+        if (w < w_end) {
+            uint4 *o = (uint4 *)(row + c * 8);
+            o[0] = make_uint4(x[0] & l0.x, x[1] & l0.y, x[2] & l0.z, x[3] & l0.w);
+            o[1] = make_uint4(x[4] & l1.x, x[5] & l1.y, x[6] & l1.z, x[7] & l1.w);
+        }
+        if (w + 32 < w_end) {
+            uint4 *o = (uint4 *)(row + (size_t)32 * L.words + c * 8);
+            o[0] = make_uint4(y[0] & l0.x, y[1] & l0.y, y[2] & l0.z, y[3] & l0.w);
+            o[1] = make_uint4(y[4] & l1.x, y[5] & l1.y, y[6] & l1.z, y[7] & l1.w);
+        }
     }
 }
 
-// Packed walk over a range [f0, f1) of the concatenated lists of a group's active units, all of
-// entry kind K (compile time).  The active units sit in lanes 0 .. n_act-1 in canonical order, with
-// strictly increasing inclusive length prefix incl (the lanes after them hold incl = total).  Each
-// pass reads 32 consecutive entries of the concatenation, one per lane: lane l takes flat entry
-// f = c0 + l, whose unit is the number of units
-// ending at or before f, counted as the units ending at or before c0 (a ballot) plus those ending
-// inside the pass (one bit each, gathered by a warp OR-reduction, then a popcount below the lane).
-// Each lane loads its entry's 2- or 4-byte key, tests the target orbital(s) in the shared orbital
-// map and queues the free entries; every 32 queued entries are evaluated at once.  Entry code =
-// list index << 5 | unit lane; a unit's list index of flat entry f is f + (list base - unit start),
-// one shuffle.  Lanes past f1 read entry 0 of the list (always allocated) and queue nothing, so the
-// test needs no bounds branch.  pos and the queues are 32-bit shared addresses.
-template <int K, typename real, typename acc_t, bool kC>
-__device__ __forceinline__ void walk_range(const ListsView &L, const View<real> &V, uint32_t f0, uint32_t f1,
-                                           uint32_t incl, uint32_t cdelta, int cmeta, int cls_row,
-                                           uint32_t *wq, int &qn, int lane, unsigned lt_mask,
-                                           int cci, int ccj, real ceinv, int cii, int cjj, acc_t &e_grp, u128 &q_grp,
-                                           unsigned &flag) {
-    const int M = V.geo.M;
-    const uint32_t sPos = (uint32_t)__cvta_generic_to_shared(V.pos);
-    uint32_t *q = K == 2 ? wq + 64 : wq;
-    const uint32_t sQ = (uint32_t)__cvta_generic_to_shared(q);
-    const uint32_t low = lane == 31 ? 0xFFFFFFFEu : ((2u << lane) - 2u);   // bits 1 .. lane
-    const uint32_t oA = K == 2 ? 0u : (uint32_t)(cls_row * M), oB = K == 2 ? (uint32_t)M : oA;
-    for (uint32_t c0 = f0; c0 < f1; c0 += 32) {
-        const uint32_t f = c0 + lane;
-        // lanes past the active units hold incl = total > c0, so they never count as "before";
-        // a unit ending at or before c0 has end = 0 (bit 0, never counted) or end >= 2^31 (no bit)
-        const unsigned before = __ballot_sync(0xffffffffu, incl <= c0);
-        const uint32_t end = incl - c0;
-        uint32_t bit;
-        asm("shl.b32 %0, 1, %1;" : "=r"(bit) : "r"(end));   // PTX clamps shifts >= 32: no bit
-        const uint32_t inside = __reduce_or_sync(0xffffffffu, bit);
-        // for valid lanes su < n_act; past f1 it may be 32, which the shuffles take modulo 32
-        const int su = __popc(before) + __popc(inside & low);
-        const bool valid = f < f1;
-        const uint32_t idx = __shfl_sync(0xffffffffu, cdelta, su) + f;   // list base - unit start + f
-        const uint32_t ridx = valid ? idx : 0u;
-        uint32_t x, y = 0xFFFFu;
-        if (K == 0) {
-            const int cls = __shfl_sync(0xffffffffu, cmeta, su) >> 2;
-            const uint32_t key = (uint32_t)__ldg(&L.s_a[ridx]);
-            asm("ld.shared.u16 %0, [%1];" : "=r"(x) : "r"(sPos + 2u * ((uint32_t)(cls * M) + (key & 0xFFFFu))));
+__global__ void __launch_bounds__(256, 5)
+k_free_bits(ListsView L, const uint32_t *__restrict__ occ_bits, int w_first, int w_end, uint32_t *__restrict__ bits) {
+    __shared__ uint2 s_occ[2 * VMC_MAX_M];
+    launch_dependents();
+    free_bits_tile(L, occ_bits, w_first, w_end, blockIdx.x, blockIdx.y, gridDim.y, bits, s_occ);
+}
+
+// The same for a batch: blockIdx.x runs over the tiles of all systems (t_begin: first tile of each).
+__global__ void __launch_bounds__(256)
+k_free_bits_batched(const SysDesc *__restrict__ sys, int n_sys) {
+    __shared__ uint2 s_occ[2 * VMC_MAX_M];
+    launch_dependents();
+    int k = 0;
+    while (k + 1 < n_sys && sys[k + 1].t_begin <= (int)blockIdx.x) ++k;
+    const SysDesc &d = sys[k];
+    free_bits_tile(d.L, d.A.occ_bits, d.w_first, d.w_first + d.w_count, blockIdx.x - d.t_begin, blockIdx.y, gridDim.y,
+                   d.bits, s_occ);
+}
+
+// One word of one walker's row, by a warp (lane = entry); ow: the walker's occupation words.
+__device__ __forceinline__ uint32_t free_word(const ListsView &L, const uint32_t *__restrict__ ow, int nw, int k, int lane) {
+    const uint32_t key = __ldg(&L.key[k * 32 + lane]);
+    const int cls = __ldg(&L.wcls[k]);
+    auto occ = [&](uint32_t p, int s) { return ow[s * nw + (p >> 5)] >> (p & 31u) & 1u; };
+    const uint32_t m = occ(key >> 16 & 0xFFu, cls & 1) & occ(key >> 24, cls >> 1) &
+                       ~(occ(key & 0xFFu, cls & 1) | occ(key >> 8 & 0xFFu, cls >> 1));
+    return __ballot_sync(0xffffffffu, m & 1u) & __ldg(&L.alive[k]);
+}
+
+// ---------------------------------------------------------------------------------- local energy
+// Exact 128-bit rate sums in two 64-bit halves (units of 2^-64).
+struct Sum128 {
+    unsigned long long lo, hi;
+    __device__ void add(unsigned long long l, unsigned long long h) {
+        lo += l;
+        hi += h + (lo < l ? 1ull : 0ull);
+    }
+};
+// Any rate, as rate_of: the general path for rates the fast ones below do not take; bit 127 tells of an
+// overflow (rates stay below 2^107).
+template <typename real> __device__ __noinline__ u128 large_rate(real ratio) {
+    unsigned flag = 0;
+    const u128 v = rate_of<real>(ratio, &flag);
+    return flag ? v | (u128)1 << 127 : v;
+}
+template <typename real> __device__ __forceinline__ void add_large_rate(Sum128 &q, real ratio, unsigned &flag) {
+    const u128 v = large_rate<real>(ratio);
+    const unsigned long long hi = (unsigned long long)(v >> 64);
+    if (hi >> 63) flag |= VMC_DEV_OVERFLOW;
+    q.add((unsigned long long)v, hi & 0x7FFFFFFFFFFFFFFFull);
+}
+// floor(|ratio| 2^64) added to q, exactly.  FP32: the integer part (below 2^32) and 2^64 times the fraction
+// are exact conversions.  FP64, below 1: the mantissa, shifted to the top of 64 bits, goes right by what the
+// exponent is below 1/2 (integer pipe: the FP64 pipe is that form's bound).
+__device__ __forceinline__ void add_rate(Sum128 &q, float ratio, unsigned &flag) {
+    const float r = fabsf(ratio);
+    if (r < 4294967296.0f) {
+        const float t = truncf(r);
+        q.add(__float2ull_rz((r - t) * 18446744073709551616.0f), (unsigned long long)__float2uint_rz(t));
+    } else {
+        add_large_rate(q, ratio, flag);
+    }
+}
+__device__ __forceinline__ void add_rate(Sum128 &q, double ratio, unsigned &flag) {
+    const unsigned long long b = abs_bits(ratio);
+    const uint32_t sh = 1022u - (uint32_t)(b >> 52);
+    if ((int)sh >= 0) {                                    // below 1
+        const unsigned long long m = (b << 11) | 0x8000000000000000ull;
+        q.add(sh < 64u ? m >> sh : 0ull, 0ull);
+    } else {
+        add_large_rate(q, ratio, flag);
+    }
+}
+// Sum over the warp: limbs of 27 bits, whose sums over 32 lanes fit 32 bits.
+__device__ __forceinline__ u128 warp_sum(const Sum128 &q) {
+    const uint32_t m = 0x7FFFFFFu;
+    const uint32_t s0 = __reduce_add_sync(0xffffffffu, (uint32_t)q.lo & m);
+    const uint32_t s1 = __reduce_add_sync(0xffffffffu, (uint32_t)(q.lo >> 27) & m);
+    const uint32_t s2 = __reduce_add_sync(0xffffffffu, (uint32_t)(q.lo >> 54 | q.hi << 10) & m);
+    const uint32_t s3 = __reduce_add_sync(0xffffffffu, (uint32_t)(q.hi >> 17) & m);
+    const uint32_t s4 = __reduce_add_sync(0xffffffffu, (uint32_t)(q.hi >> 44));
+    return (u128)s0 + ((u128)s1 << 27) + ((u128)s2 << 54) + ((u128)s3 << 81) + ((u128)s4 << 108);
+}
+
+// Per spin orbital, in shared memory: exp(S) of an empty one with the element offset of its G row from
+// the first alpha row; 1/exp(S) of a filled one with its column.
+template <typename real> struct OrbTable;
+template <> struct OrbTable<float> {
+    float2 *t;
+    static constexpr size_t bytes = 8;
+    __device__ OrbTable(void *p, int) : t((float2 *)p) {}
+    __device__ void set(int p, float e, int off) { t[p] = make_float2(e, __int_as_float(off)); }
+    __device__ float e(int p) const { return t[p].x; }
+    __device__ int off(int p) const { return __float_as_int(t[p].y); }
+    __device__ void get(int p, float &e, int &off) const {
+        const float2 v = t[p];
+        e = v.x;
+        off = __float_as_int(v.y);
+    }
+};
+// (with scaled G rows the entries read the offsets alone)
+template <> struct OrbTable<double> {
+    double *e_;
+    int *off_;
+    static constexpr size_t bytes = 12;
+    __device__ OrbTable(void *p, int n) : e_((double *)p), off_((int *)((double *)p + n)) {}
+    __device__ void set(int p, double e, int off) { e_[p] = e; off_[p] = off; }
+    __device__ double e(int p) const { return e_[p]; }
+    __device__ void get(int p, double &e, int &off) const { e = e_[p]; off = off_[p]; }
+    __device__ int off(int p) const { return off_[p]; }
+};
+
+// Value of flat entry e (a move of this walker): returns H_nm and the ratio, adds the rate to q.
+// K: 0 single, 1 same-spin double, 2 opposite-spin double, 3 either double (second: a same-spin one,
+// whose minor has a second product); sa, sb: M if the spin of (a, i), (b, j) is beta; valid: the lane has
+// an entry of its own (the others repeat one and count nothing); key_out: the key (singles: spin orbital i);
+// scaled: G[a][i] holds G_ai E_a / E_i.
+// The rounding is entry_value's.  The FP64 form multiplies E_a / E_i into G once per walker and element
+// (two products each, 12.8 K elements at H160) instead of four products per entry: GB300 has 2 FP64
+// multiply-adds per clock and SM, so a batch of 32 spends 16 clocks on every one.  It pays with long lists (rule in
+// lists.cu): without doubles the two products per element are what costs.
+template <int K, typename real, bool kC, bool scaled>
+__device__ __forceinline__ real flat_value(const ListsView &L, const View<real> &V, const OrbTable<real> &orb, uint32_t e,
+                                           int sa, int sb, bool second, bool valid, Sum128 &q, unsigned &flag, real &ratio, uint32_t &key_out) {
+    const auto r = flat_rec(L, e, real(0));
+    const uint32_t key = low_bits(r.x);
+    key_out = key;
+    const real *G = V.Ga;
+    real ea, ei, rt, h;
+    int ra, ci;
+    if (K == 0) {
+        const uint32_t aux = low_bits(r.w);
+        const int s = aux >= (uint32_t)L.ns_pad ? V.geo.M : 0, A = s + (int)(key & 0xFFu), I = s + (int)(key >> 24);
+        key_out = (uint32_t)I;
+        if (scaled) { ra = orb.off(A); ci = orb.off(I); }
+        else { orb.get(A, ea, ra); orb.get(I, ei, ci); }
+        rt = rmul(G[ra + ci], r.z);
+        if (!scaled) rt = rmul(rmul(rt, ea), ei);
+        if (kC) rt = rmul(rt, cps_ratio<real>(V, I, A, I, A, 2));
+        h = V.F[aux];
+    } else {
+        const int A = sa + (int)(key & 0xFFu), B = sb + (int)(key >> 8 & 0xFFu);
+        const int I = sa + (int)(key >> 16 & 0xFFu), J = sb + (int)(key >> 24);
+        real eb, ej;
+        int rb, cj;
+        if (scaled) {
+            ra = orb.off(A); rb = orb.off(B); ci = orb.off(I); cj = orb.off(J);
         } else {
-            const uint32_t key = __ldg((K == 2 ? L.do_ab : L.ds_ab) + ridx);
-            asm("ld.shared.u16 %0, [%1];" : "=r"(x) : "r"(sPos + 2u * (oA + (key & 0xFFFFu))));
-            asm("ld.shared.u16 %0, [%1];" : "=r"(y) : "r"(sPos + 2u * (oB + (key >> 16))));
+            orb.get(A, ea, ra); orb.get(B, eb, rb); orb.get(I, ei, ci); orb.get(J, ej, cj);
         }
-        const bool pass = valid && (x & y & 0x8000u);
-        const unsigned bal = __ballot_sync(0xffffffffu, pass);
-        if (pass)
-            asm volatile("st.shared.u32 [%0], %1;" ::"r"(sQ + 4u * (uint32_t)(qn + __popc(bal & lt_mask))),
-                         "r"((idx << 5) | (uint32_t)su) : "memory");
-        qn += __popc(bal);
-        if (qn >= 32) {
-            __syncwarp();
-            qn -= 32;
-            drain_queue<K, real, acc_t, kC>(L, V, q + qn, 32, lane, cci, ccj, ceinv, cmeta, cii, cjj, e_grp, q_grp,
-                                            flag);
-            __syncwarp();
-        }
+        real x;
+        if (K == 1 || (K == 3 && second)) x = minor2(G[ra + ci], G[rb + cj], G[ra + cj], G[rb + ci]);
+        else x = rmul(G[ra + ci], G[rb + cj]);
+        rt = rmul(x, r.z);
+        if (!scaled) rt = rmul(rmul(rmul(rt, ea), eb), rmul(ei, ej));
+        if (kC) rt = rmul(rt, cps_ratio<real>(V, I, A, J, B, 4));
+        h = r.y;
     }
+    if (!valid) rt = real(0);
+    add_rate(q, rt, flag);
+    ratio = rt;
+    return h;
 }
 
-// Local energy of walker w by the whole CTA (any number of warps).  smraw: dynamic shared memory.
-template <typename real, bool kC>
+// Shared memory of one warp: codes (entry position in the block) of free entries.  32 places before and
+// behind the codes may be read: batches are full reads.
+constexpr int kFreeMax = 160;
+struct WarpBuf {
+    uint16_t pad[32], code[kFreeMax + 32];
+};
+
+// Running sum of the mixed form's FP32 energy contributions of one group and kind, in a fixed order:
+// the entries of the occupied units form windows of 32 places (free or not); after each window its free
+// entries go on a stack, and as soon as the stack holds 32 or more the top 32 are added, lane l the
+// l-th from below; what is left at the end is added by lanes 0 .. q-1.  Free entries arrive in batches of 32,
+// one per lane, with their places.  With a batch the previous full one can be added: the window that
+// filled the stack is that of the previous batch's last entry, and q of the new entries lie in
+// it too and are what the addition leaves on the stack.  So lanes >= q take the stack (below) and the
+// previous batch, lanes < q the new one, rotated by q.
+struct StackSum {
+    float below = 0.f, last = 0.f;   // the stack's contributions; the previous batch
+    int q = 0, n_last = 0;           // entries on the stack; entries of the previous batch (0: none yet)
+    uint32_t place = 0;              // places of the previous batch's entries
+    __device__ void drain(int qn, float c, int lane, float &acc) {
+        const float m = lane < q ? below : last;
+        acc += __shfl_sync(0xffffffffu, lane >= qn ? m : c, (lane + qn) & 31);
+        below = m;
+        q = qn;
+    }
+    // a batch of n <= 32 entries (lanes < n; only the last one has n < 32): contributions c, places p
+    __device__ void batch(float c, uint32_t p, int n, int lane, float &acc) {
+        if (n_last) {
+            const uint32_t end = __shfl_sync(0xffffffffu, place, 31) | 31u;      // the window's last place
+            const unsigned after = __ballot_sync(0xffffffffu, lane >= n || p > end);
+            drain(after ? __ffs(after) - 1 : 32, c, lane, acc);
+        }
+        place = p;
+        last = c;
+        n_last = n;
+    }
+    // after the last batch: its own addition if it was full, else what this lane has still to add
+    __device__ float finish(int lane, float &acc) {
+        if (n_last == 32) {
+            drain(0, 0.f, lane, acc);
+            return 0.f;
+        }
+        return lane < n_last ? (lane < q ? below : last) : 0.f;
+    }
+};
+
+// Local energy of walker w by the whole CTA (any number of warps).  row: the walker's free-entry bits
+// (null: made here); smraw: dynamic shared memory.
+//
+// Warps take the groups dynamically; each group's sums are stored by index, so the result does not depend on
+// which warp took it.  A group's free entries are the set bits of a contiguous range of the row: a lane
+// reads two words, a popcount prefix ranks its bits, and it writes their positions to the warp's code
+// buffer; 32 at a time, one per lane, they are evaluated (flat_value).  Nothing is done for entries that
+// are not free: the first version of this walk loaded and tested each of the ~62 K entries of an H160
+// walker's occupied pairs to find its 13 K moves, and more than half of its instructions were that test.
+// FP64 form: batches run over both kinds of a group.  Mixed form: the kinds are kept apart and the FP32
+// sums keep the fixed order of StackSum; an entry's place counts the entries of occupied units only, from the
+// unit table.
+template <typename real, bool kC, bool scaled>
 __device__ __forceinline__ void eloc_walker(const ListsView &L, const WalkerArgs &A, const int w,
-                                            double *__restrict__ e_loc, double *__restrict__ t_res,
-                                            u128 *__restrict__ rates, unsigned *status, unsigned char *smraw,
-                                            const CpsView &C = CpsView{}) {
+                                            const uint32_t *__restrict__ row, double *__restrict__ e_loc,
+                                            double *__restrict__ t_res, u128 *__restrict__ rates, unsigned *status,
+                                            unsigned char *smraw, const CpsView &C = CpsView{}) {
+    constexpr bool kOrder = sizeof(real) == 4;
     const Geo geo = make_geo(A.M, A.na, A.nb);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x, nwarp = nt >> 5;
-    const int M = geo.M, n_groups = L.n_groups, n_sgl_groups = (2 * M + 31) / 32;
+    const int M = geo.M, nw = geo.nw, n_groups = L.n_groups, n_sgl_groups = (2 * M + 31) / 32;
     const int lda = geo.na + 1, ldb = geo.nb + 1;    // padded rows: no bank conflicts on columns
-    real *sGa = (real *)smraw;
-    real *sGb = sGa + (size_t)geo.nv_a * lda;
-    real *sE = sGb + (size_t)geo.nv_b * ldb;
-    uint16_t *pos = (uint16_t *)(sE + 2 * M);
-    // per-group energy partials: global, after the system's rate sums (written and read by this CTA)
-    double *eg = (double *)(rates + (size_t)A.W * n_groups) + (size_t)w * n_groups;
-    // per warp: two queues of 64 entry codes (idx << 5 | unit lane): kinds 0/1, and kind 2
-    uint32_t *wq = (uint32_t *)(((uintptr_t)(pos + 2 * M) + 15) & ~(uintptr_t)15) + warp * 128;
-    // correlator product, after the queues: 1 / c_l[n_l], the current coefficient positions and
+    real *sG = (real *)smraw;
+    const size_t g_el = (size_t)geo.nv_a * lda + (size_t)geo.nv_b * ldb;
+    // (offsets from smraw, so that every access stays a shared-memory instruction)
+    const size_t o_orb = (g_el * sizeof(real) + 7) & ~(size_t)7, o_occ = o_orb + OrbTable<real>::bytes * (size_t)(2 * M);
+    const size_t o_row = (o_occ + sizeof(uint32_t) * 2 * nw + 15) & ~(size_t)15;
+    const size_t o_buf = o_row + (row ? 0 : sizeof(uint32_t) * (size_t)L.words);   // (words: a multiple of 8)
+    OrbTable<real> orb(smraw + o_orb, 2 * M);
+    typedef WarpBuf Buf;
+    uint32_t *s_occ = (uint32_t *)(smraw + o_occ);   // [2 nw] the walker's occupation words
+    uint32_t *s_row = (uint32_t *)(smraw + o_row);   // the walker's free-entry bits if row is null
+    Buf *bufs = (Buf *)(smraw + o_buf);
+    Buf &wb = bufs[warp];
+    // correlator product, after the warp buffers: 1 / c_l[n_l], the current coefficient positions and
     // the coefficient offsets
-    real *sCinv = (real *)((uint32_t *)(((uintptr_t)(pos + 2 * M) + 15) & ~(uintptr_t)15) + nwarp * 128);
+    real *sCinv = (real *)(bufs + nwarp);
     int32_t *sCur = (int32_t *)(sCinv + ((C.n_corr + 3) & ~3));
     int32_t *sVoff = sCur + C.n_corr;
-    __shared__ u128 red_q[32];
+    // per-group energy partials: global, after the system's rate sums (written and read by this CTA)
+    double *eg = (double *)(rates + (size_t)A.W * n_groups) + (size_t)w * n_groups;
     __shared__ int next_group;
 
     // ---- prologue: stage G into padded rows, exp(S), orbital map
     {
+        // the walker's bits are read group by group: bring them to L2 while the tables are staged
+        if (tid == 0 && row && L.words > 0)
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(row), "r"(4u * (uint32_t)L.words) : "memory");
         const real *Gw = (const real *)A.G + (size_t)w * geo.g_stride;
         const size_t na_el = (size_t)geo.nv_a * geo.na;
-        for (int r = warp; r < geo.nv_a + geo.nv_b; r += nwarp) {   // one row per warp
-            const bool bs = r >= geo.nv_a;
-            const int rr = bs ? r - geo.nv_a : r, n = bs ? geo.nb : geo.na;
-            const real *src = Gw + (bs ? na_el + (size_t)rr * geo.nb : (size_t)rr * geo.na);
-            real *dst = bs ? sGb + (size_t)rr * ldb : sGa + (size_t)rr * lda;
-            for (int c = lane; c < n; c += 32) dst[c] = src[c];
+        real *sGb = sG + (size_t)geo.nv_a * lda;
+        if constexpr (!scaled) {
+            // one row per warp, asynchronous copies (all of a thread's in flight; the odd row stride
+            // leaves pieces of one element)
+            for (int r = warp; r < geo.nv_a + geo.nv_b; r += nwarp) {
+                const bool bs = r >= geo.nv_a;
+                const int rr = bs ? r - geo.nv_a : r, n = bs ? geo.nb : geo.na;
+                const real *src = Gw + (bs ? na_el + (size_t)rr * geo.nb : (size_t)rr * geo.na);
+                const uint32_t dst = (uint32_t)__cvta_generic_to_shared(bs ? sGb + (size_t)rr * ldb : sG + (size_t)rr * lda);
+                for (int c = lane; c < n; c += 32)
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(dst + (uint32_t)(c * sizeof(real))), "l"(src + c),
+                                 "n"(sizeof(real)) : "memory");
+            }
+        }
+        if (!row) {
+            const uint32_t *ow = A.occ_bits + (size_t)w * 2 * nw;
+            for (int k = warp; k < L.words; k += nwarp) {
+                const uint32_t x = free_word(L, ow, nw, k, lane);
+                if (lane == 0) s_row[k] = x;
+            }
         }
         const real *Sw = (const real *)A.S + (size_t)w * 2 * M;
         const uint16_t *pw = A.pos + (size_t)w * 2 * M;
         for (int p = tid; p < 2 * M; p += nt) {
-            const uint16_t ps = pw[p];
+            const int ps = pw[p];
             const real e = rexp(Sw[p]);
-            sE[p] = (ps & 0x8000) ? e : rrcp(e);
-            pos[p] = ps;
+            if (ps & 0x8000) orb.set(p, e, (ps & 0x7FFF) * (p < M ? lda : ldb) + (p < M ? 0 : geo.nv_a * lda));
+            else orb.set(p, rrcp(e), ps);
         }
+        if constexpr (scaled) {
+            // rows scaled by E of their orbital and 1/E of their columns'; four rows per warp at a time
+            __syncthreads();
+            const uint16_t *occ = A.occ_list + (size_t)w * geo.ne, *virt = A.virt_list + (size_t)w * (2 * M - geo.ne);
+            for (int s = 0; s < 2; ++s) {
+                const int n = geo.n(s), nv = M - n, ld = s ? ldb : lda;
+                const real *src = Gw + (s ? na_el : 0);
+                real *dst = s ? sGb : sG;
+                for (int c = lane; c < n; c += 32) {
+                    const real ec = orb.e(s * M + occ[(s ? geo.na : 0) + c]);
+                    for (int r0 = warp; r0 < nv; r0 += 4 * nwarp) {
+                        real g[4];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) g[k] = r0 + k * nwarp < nv ? src[(size_t)(r0 + k * nwarp) * n + c] : real(0);
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const int r = r0 + k * nwarp;
+                            if (r < nv) dst[(size_t)r * ld + c] = rmul(rmul(g[k], orb.e(s * M + virt[(s ? geo.nv_a : 0) + r])), ec);
+                        }
+                    }
+                }
+            }
+        }
+        for (int t = tid; t < 2 * nw; t += nt) s_occ[t] = A.occ_bits[(size_t)w * 2 * nw + t];
         if (kC) {
             for (int l = tid; l <= C.n_corr; l += nt) sVoff[l] = C.val_off[l];
             for (int l = tid; l < C.n_corr; l += nt) {
@@ -492,112 +737,183 @@ __device__ __forceinline__ void eloc_walker(const ListsView &L, const WalkerArgs
             }
         }
         if (tid == 0) next_group = nwarp;
+        if (!scaled) asm volatile("cp.async.wait_all;" ::: "memory");
+        if (row) wait_dependency();      // the rows (a kernel may still be writing them)
     }
     __syncthreads();
 
     View<real> V;
-    V.pos = pos; V.Ga = sGa; V.Gb = sGb; V.lda = lda; V.ldb = ldb;
-    V.E = sE; V.S = nullptr; V.F = (const real *)A.F + (size_t)w * 2 * L.ns_pad; V.geo = geo;
+    V.Ga = sG; V.F = (const real *)A.F + (size_t)w * 2 * L.ns_pad; V.geo = geo;
     V.C = C; V.voff = sVoff; V.cur = sCur; V.cidx = nullptr; V.cinv = sCinv;
     typedef typename AccT<real>::type acc_t;
-    u128 q_tot = 0;
     unsigned flag = 0;
 
-    // Groups are taken dynamically; each group's sums are stored by index, so the result does not
-    // depend on which warp took it.  Inside a group the warp walks the units' lists with a cheap
-    // key check and queues the entries whose targets are free; the ratio, rate and energy of
-    // queued entries are evaluated 32 at a time, one per lane, so that work is never divergent.
-    const unsigned lt_mask = (1u << lane) - 1u;
     for (int g = warp; g < n_groups;) {
-        Unit<real> u;
-        const bool act = setup_unit<real>(L, V, g, lane, u);
+        const uint4 gi = __ldg(&L.group[g]);             // first word, first opposite-spin word, end, spin
+        const bool pairs = g >= n_sgl_groups;
         acc_t e_grp = 0;
-        u128 q_grp = 0;
-        unsigned amask = __ballot_sync(0xffffffffu, act);
-        if (__ballot_sync(0xffffffffu, act && u.base + u.len > list_size(L, u.kind))) {   // cannot happen: guard
-            flag |= VMC_DEV_INCONSISTENT;
-            amask = 0;
-        }
-        const int n_act = __popc(amask);
-        if (n_act == 0) {                // an empty group (its row orbital unoccupied): zero sums
-            if (lane == 0) {
-                rates[(size_t)w * n_groups + g] = 0;
-                eg[g] = 0.0;
+        Sum128 q{0, 0};
+        bool any = false;
+        uint32_t to_place = 0;                           // mixed form: place - flat entry of unit `lane`
+        StackSum sum;
+        float restA = 0.f;                               // what the same-spin part left to add
+        bool in_a = true;
+        uint32_t carry_e = 0;                            // entries waiting for a full batch (lanes < n_carry)
+        int n_carry = 0;
+        for (uint32_t w0 = gi.x; w0 < gi.z;) {
+            const uint32_t wi = w0 + 2 * lane;
+            uint2 x = make_uint2(0u, 0u);
+            if (wi < gi.z) {
+                x = row ? *(const uint2 *)(row + wi) : *(const uint2 *)(s_row + wi);
+                if (wi + 1 >= gi.z) x.y = 0;
             }
-            int nxt = 0;
-            if (lane == 0) nxt = atomicAdd(&next_group, 1);
-            g = __shfl_sync(0xffffffffu, nxt, 0);
-            continue;
-        }
-        // compact the active units into lanes 0 .. n_act-1, in order (same-spin units precede the
-        // opposite-spin ones of a row); the queue, empty between groups, holds the permutation
-        const int n1 = __popc(amask & __ballot_sync(0xffffffffu, u.kind != 2));
-        if ((amask >> lane) & 1u) wq[__popc(amask & lt_mask)] = (uint32_t)lane;
-        __syncwarp();
-        const int src = lane < n_act ? (int)wq[lane] : lane;
-        __syncwarp();
-        const uint32_t clen0 = __shfl_sync(0xffffffffu, u.len, src);
-        const uint32_t clen = lane < n_act ? clen0 : 0u;
-        const uint32_t cbase = __shfl_sync(0xffffffffu, u.base, src);
-        const int cmeta = __shfl_sync(0xffffffffu, u.kind | (u.cls << 2), src);
-        const int cci = __shfl_sync(0xffffffffu, u.ci, src), ccj = __shfl_sync(0xffffffffu, u.cj, src);
-        const int cii = kC ? __shfl_sync(0xffffffffu, u.i, src) : 0, cjj = kC ? __shfl_sync(0xffffffffu, u.j, src) : 0;
-        const real ceinv = __shfl_sync(0xffffffffu, u.einv, src);
-        // inclusive prefix of the compacted list lengths; t1 = end of the same-spin (or singles) part
-        uint32_t incl = clen;
+            if (!__any_sync(0xffffffffu, x.x | x.y) && n_carry == 0) {
+                w0 += 64;
+                continue;
+            }
+            const uint32_t blk = w0 * 32;
+            const uint32_t f0 = __popc(x.x), own = f0 + __popc(x.y);
+            if constexpr (kOrder) {
+                // first block with free entries: the units, for the places of a kind's entries, which its second
+                // batch needs.  A long group will have one; a short one (one block) is counted first.
+                bool need = !any;
+                if (need && gi.z - gi.x <= 20u) {
+                    const uint32_t fA = (wi < gi.y ? f0 : 0u) + (wi + 1 < gi.y ? own - f0 : 0u);
+                    const uint32_t c = __reduce_add_sync(0xffffffffu, fA << 16 | (own - fA));
+                    need = max(c >> 16, c & 0xFFFFu) > 32u;
+                }
+                if (need) {
+                    const uint4 t = __ldg(&L.unit_tab[(size_t)g * 32 + lane]);
+                    const int kind = (int)(t.w & 3u), sp = (int)(t.w >> 2);
+                    const uint32_t i = t.x & 0xFFFFu, j = kind == 0 ? i : t.x >> 16;
+                    const uint32_t bi = s_occ[(kind == 2 ? 0 : sp * nw) + (i >> 5)] >> (i & 31u);
+                    const uint32_t bj = s_occ[(kind == 2 ? nw : sp * nw) + (j >> 5)] >> (j & 31u);
+                    const uint32_t len = (bi & bj & 1u) ? t.z : 0u;
+                    uint32_t us = len;
 #pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const uint32_t o = __shfl_up_sync(0xffffffffu, incl, d);
-            if (lane >= d) incl += o;
-        }
-        const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
-        const uint32_t cdelta = cbase - (incl - clen);   // list index of flat entry f: f + cdelta (mod 2^32)
-        const uint32_t t1v = __shfl_sync(0xffffffffu, incl, n1 > 0 ? n1 - 1 : 0), t1 = n1 > 0 ? t1v : 0u;
-        const int cls_row = __shfl_sync(0xffffffffu, cmeta, 0) >> 2;   // spin of a row group's same-spin units
-        int qn0 = 0, qn1 = 0;   // queue fill (warp-uniform)
-        if (g < n_sgl_groups) {
-            walk_range<0, real, acc_t, kC>(L, V, 0, total, incl, cdelta, cmeta, 0, wq, qn0, lane, lt_mask,
-                                           cci, ccj, ceinv, cii, cjj, e_grp, q_grp, flag);
+                    for (int d = 1; d < 32; d <<= 1) {
+                        const uint32_t o = __shfl_up_sync(0xffffffffu, us, d);
+                        if (lane >= d) us += o;
+                    }
+                    // (same-spin units stand before the opposite-spin ones)
+                    const uint32_t uA = __reduce_max_sync(0xffffffffu, kind != 2 && t.z ? us : 0u);
+                    to_place = us - len - (kind == 2 ? uA : 0u) - t.y;
+                }
+            }
+            any = true;
+            uint32_t sc = own;                           // free entries up to and with the lane's words
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t o = __shfl_up_sync(0xffffffffu, sc, d);
+                if (lane >= d) sc += o;
+            }
+            // lanes of this block whose codes fit the buffer
+            const int nl = __popc(__ballot_sync(0xffffffffu, sc <= (uint32_t)kFreeMax));
+            const uint32_t at0 = sc - own;
+            if (lane < nl) {
+                uint16_t *at = wb.code + at0;
+#pragma unroll 1
+                for (uint32_t y = x.x; y; y &= y - 1u) *at++ = (uint16_t)(lane << 6 | (__ffs(y) - 1));
+#pragma unroll 1
+                for (uint32_t y = x.y; y; y &= y - 1u) *at++ = (uint16_t)(lane << 6 | 32 | (__ffs(y) - 1));
+            }
             __syncwarp();
-            if (qn0)
-                drain_queue<0, real, acc_t, kC>(L, V, wq, qn0, lane, cci, ccj, ceinv, cmeta, cii, cjj, e_grp, q_grp,
-                                                flag);
-        } else {
-            walk_range<1, real, acc_t, kC>(L, V, 0, t1, incl, cdelta, cmeta, cls_row, wq, qn0, lane, lt_mask,
-                                           cci, ccj, ceinv, cii, cjj, e_grp, q_grp, flag);
-            walk_range<2, real, acc_t, kC>(L, V, t1, total, incl, cdelta, cmeta, cls_row, wq, qn1, lane,
-                                           lt_mask, cci, ccj, ceinv, cii, cjj, e_grp, q_grp, flag);
+            const int n = (int)__reduce_max_sync(0xffffffffu, lane < nl ? sc : 0u);
+            const uint32_t w1 = w0 + 2 * (uint32_t)nl;
+            const bool done = w1 >= gi.z;
+            // the carried entries and the codes s0 .. s1-1, 32 at a time; end: the last, partly filled
+            // batch too (otherwise it is carried)
+            auto batches = [&](auto kind, int s0, int s1, bool end) {
+                constexpr int K = decltype(kind)::value;
+                const int total = n_carry + s1 - s0;
+                int t0 = 0;
+                for (; t0 < total; t0 += 32) {
+                    const int t = t0 + lane, cnt = min(32, total - t0);
+                    // (lanes outside the codes read a neighbouring place of the warp's buffer)
+                    const uint32_t c = wb.code[s0 - n_carry + t] & 2047u;
+                    uint32_t e = blk + c;
+                    if (t < n_carry) e = carry_e;
+                    if (cnt < 32) {
+                        if (!end) {
+                            carry_e = e;
+                            break;
+                        }
+                        const uint32_t e0 = __shfl_sync(0xffffffffu, e, 0);
+                        if (lane >= cnt) e = e0;
+                    }
+                    real rt;
+                    uint32_t key;
+                    const bool opp = K == 2 || (K == 3 && (e >> 5) >= gi.y), beta = (K == 1 || K == 3) && (gi.w & 1u);
+                    const real h = flat_value<K, real, kC, scaled>(L, V, orb, e, beta ? M : 0, (opp || beta) ? M : 0, !opp,
+                                                           lane < cnt, q, flag, rt, key);
+                    if constexpr (kOrder) {
+                        // the lane of the entry's unit, modulo 32 (ListsView::group)
+                        const uint32_t j = key >> 24, i = key >> 16 & 0xFFu;
+                        const uint32_t un = K == 0 ? key : (K == 1 ? j + i * (gi.w >> 1 & 31u) + (gi.w >> 6) : j + (gi.w >> 11));
+                        const uint32_t place = e + __shfl_sync(0xffffffffu, to_place, (int)(un & 31u));
+                        sum.batch(rmul(h, rt), place, cnt, lane, e_grp);
+                    } else {
+                        e_grp = __fma_rn(lane < cnt ? h : real(0), rt, e_grp);
+                    }
+                }
+                n_carry = max(0, total - t0);
+            };
+            if (!pairs) {
+                batches(std::integral_constant<int, 0>{}, 0, n, done);
+            } else if constexpr (!kOrder) {
+                batches(std::integral_constant<int, 3>{}, 0, n, done);
+            } else {
+                int nA = 0;                              // codes of the block's same-spin part
+                if (gi.y > w0) {
+                    const uint32_t ws = gi.y - w0, l2 = 2 * (uint32_t)lane;      // words before the opposite-spin part
+                    nA = (int)__reduce_max_sync(0xffffffffu, lane >= nl || l2 >= ws ? 0u : (l2 + 1 < ws ? sc : at0 + f0));
+                    batches(std::integral_constant<int, 1>{}, 0, nA, w1 >= gi.y);
+                }
+                if (w1 > gi.y) {
+                    if (in_a) {
+                        restA = sum.finish(lane, e_grp);
+                        sum = StackSum{};
+                        in_a = false;
+                    }
+                    batches(std::integral_constant<int, 2>{}, nA, n, done);
+                }
+            }
             __syncwarp();
-            if (qn0)
-                drain_queue<1, real, acc_t, kC>(L, V, wq, qn0, lane, cci, ccj, ceinv, cmeta, cii, cjj, e_grp, q_grp,
-                                                flag);
-            if (qn1)
-                drain_queue<2, real, acc_t, kC>(L, V, wq + 64, qn1, lane, cci, ccj, ceinv, cmeta, cii, cjj, e_grp,
-                                                q_grp, flag);
+            w0 = w1;
         }
-        __syncwarp();
-        const double eg_sum = warp_sum_acc(e_grp);   // FP32 lanes in the mixed form: one conversion
-        q_grp = warp_sum_u128(q_grp);
+        if constexpr (kOrder) {
+            const float rest = sum.finish(lane, e_grp);
+            e_grp += restA;
+            e_grp += rest;
+        }
+        u128 q_grp = 0;
+        double eg_sum = 0.0;
+        if (any) {
+            eg_sum = warp_sum_acc(e_grp);   // FP32 lanes in the mixed form: one conversion
+            q_grp = warp_sum(q);
+        }
+        int nxt = 0;
         if (lane == 0) {
             rates[(size_t)w * n_groups + g] = q_grp;
             eg[g] = eg_sum;
+            nxt = atomicAdd(&next_group, 1);
         }
-        q_tot += q_grp;
-        int nxt = 0;
-        if (lane == 0) nxt = atomicAdd(&next_group, 1);
         g = __shfl_sync(0xffffffffu, nxt, 0);
     }
-    if (lane == 0) red_q[warp] = q_tot;
     if (flag) atomicOr(status, flag);
     __syncthreads();
     if (warp == 0) {
-        // fixed-order sum of the per-group energies: lane l takes groups l, l+32, ...
+        // sums over the groups: the energies in a fixed order (lane l takes groups l, l+32, ...), the
+        // rates exactly
         double s = 0.0;
-        for (int g = lane; g < n_groups; g += 32) s += eg[g];
+        u128 Q = 0;
+        for (int g = lane; g < n_groups; g += 32) {
+            s += eg[g];
+            Q += rates[(size_t)w * n_groups + g];
+        }
         s = warp_sum_f64(s);
+        Q = warp_sum_u128(Q);
         if (lane == 0) {
-            u128 Q = 0;
-            for (int k = 0; k < nwarp; ++k) Q += red_q[k];
             e_loc[w] = A.e_diag[w] + s;
             if (Q == 0) {
                 t_res[w] = 0.0;
@@ -616,22 +932,24 @@ __device__ __forceinline__ void eloc_walker(const ListsView &L, const WalkerArgs
 // memory (the walker's G rows) rather than registers bounds the CTAs per SM.
 template <int kT> struct EmB { static constexpr int v = kT >= 512 ? 2 : (kT >= 384 ? 3 : (kT >= 256 ? 4 : 8)); };
 
-template <typename real, int kT>
+template <typename real, int kT, bool kS>
 __global__ void __launch_bounds__(kT, EmB<kT>::v)
-k_local_energy(ListsView L, WalkerArgs A, double *__restrict__ e_loc, double *__restrict__ t_res,
-               u128 *__restrict__ rates, unsigned *status) {
+k_local_energy(ListsView L, WalkerArgs A, int w_first, const uint32_t *__restrict__ bits, double *__restrict__ e_loc,
+               double *__restrict__ t_res, u128 *__restrict__ rates, unsigned *status) {
     extern __shared__ __align__(16) unsigned char smraw[];
-    eloc_walker<real, false>(L, A, blockIdx.x, e_loc, t_res, rates, status, smraw);
+    eloc_walker<real, false, kS>(L, A, w_first + blockIdx.x, bits ? bits + (size_t)blockIdx.x * L.words : nullptr, e_loc,
+                             t_res, rates, status, smraw);
 }
 
 // The same with the correlator product (a separate instantiation, so the pair-Jastrow kernel above
 // is not touched by it).
-template <typename real, int kT>
+template <typename real, int kT, bool kS>
 __global__ void __launch_bounds__(kT, EmB<kT>::v)
-k_local_energy_cps(ListsView L, WalkerArgs A, CpsView C, double *__restrict__ e_loc, double *__restrict__ t_res,
-                   u128 *__restrict__ rates, unsigned *status) {
+k_local_energy_cps(ListsView L, WalkerArgs A, CpsView C, int w_first, const uint32_t *__restrict__ bits,
+                   double *__restrict__ e_loc, double *__restrict__ t_res, u128 *__restrict__ rates, unsigned *status) {
     extern __shared__ __align__(16) unsigned char smraw[];
-    eloc_walker<real, true>(L, A, blockIdx.x, e_loc, t_res, rates, status, smraw, C);
+    eloc_walker<real, true, kS>(L, A, w_first + blockIdx.x, bits ? bits + (size_t)blockIdx.x * L.words : nullptr, e_loc,
+                            t_res, rates, status, smraw, C);
 }
 
 // Batched launch over several systems (uneven sizes).  CTAs stay resident and take walkers from
@@ -650,19 +968,29 @@ k_local_energy_batched(const SysDesc *__restrict__ sys, int n_sys, int total, in
         int k = 0;
         while (k + 1 < n_sys && sys[k + 1].w_begin <= t) ++k;
         const SysDesc &d = sys[k];
-        eloc_walker<real, false>(d.L, d.A, t - d.w_begin, d.e_loc, d.t_res, d.rates, status, smraw);
+        const int l = t - d.w_begin;
+        const uint32_t *row = d.bits + (size_t)l * d.L.words;
+        if (sizeof(real) == 8 && d.L.scaled)
+            eloc_walker<real, false, sizeof(real) == 8>(d.L, d.A, d.w_first + l, row, d.e_loc, d.t_res, d.rates, status, smraw);
+        else
+            eloc_walker<real, false, false>(d.L, d.A, d.w_first + l, row, d.e_loc, d.t_res, d.rates, status, smraw);
     }
 }
 
 // ---------------------------------------------------------------------------------- CTMC
 // Selection: one warp per walker.  Scans the walker's group sums (u128), draws Philox, finds the
-// group whose prefix crosses T and re-walks only that group with the same entry code as the
-// local-energy kernel.  Writes the move code (0 = no move) and advances the walker's counter.
+// group whose prefix crosses T and evaluates only that group's free entries, 32 at a time in canonical
+// order, with the values of the local-energy kernel.  Writes the move code (0 = no move) and advances the
+// walker's counter.  The free entries come from the rows of bits that the local energy left (row), or
+// are found here, a word of 32 entries per step (null).  A warp per walker has nothing to hide its
+// latency behind in a small call, so what counts is the number of dependent steps: one per 32 free
+// entries instead of one per occupied unit (256 walkers of the 10-site ring: 36 -> 26 us for choice and
+// update).
 template <typename real, bool kC>
 __device__ __forceinline__ void select_walker(const ListsView &L, const WalkerArgs &A, const int w,
-                                              const u128 *__restrict__ rates, uint64_t seed,
-                                              uint64_t *__restrict__ move_code, unsigned *status,
-                                              const CpsView &C = CpsView{}) {
+                                              const u128 *__restrict__ rates, const uint32_t *__restrict__ row,
+                                              uint64_t seed, uint64_t *__restrict__ move_code, unsigned *status,
+                                              WarpBuf &wb, const CpsView &C = CpsView{}) {
     const Geo geo = make_geo(A.M, A.na, A.nb);
     const int lane = threadIdx.x & 31;
     const int M = geo.M, N2 = 2 * M, n_groups = L.n_groups;
@@ -700,39 +1028,56 @@ __device__ __forceinline__ void select_walker(const ListsView &L, const WalkerAr
         V.pos = A.pos + (size_t)w * N2; V.Ga = Gw; V.Gb = Gw + geo.g_off(1); V.lda = geo.na; V.ldb = geo.nb;
         V.E = nullptr; V.S = Sw; V.F = (const real *)A.F + (size_t)w * 2 * L.ns_pad; V.geo = geo;
         if (kC) cps_global(V, C, A.cps + (size_t)w * C.n_corr);
-        Unit<real> u;
-        const bool act = setup_unit<real>(L, V, gsel, lane, u);
-        unsigned mask = __ballot_sync(0xffffffffu, act);
+        const uint4 gi = __ldg(&L.group[gsel]);
+        const bool single = gsel < (N2 + 31) / 32;
+        const uint32_t *ow = A.occ_bits + (size_t)w * 2 * geo.nw;
         u128 carry = 0;
         unsigned flag = 0;
         bool found = false;
-        while (mask && !found) {
-            const int src = __ffs(mask) - 1;
-            mask &= mask - 1;
-            const Unit<real> v = shfl_unit(u, src);
-            for (uint32_t k0 = 0; k0 < v.len && !found; k0 += 32) {
-                const uint32_t k = k0 + lane;
+        for (uint32_t w0 = gi.x; w0 < gi.z && !found;) {
+            // 32 words of the group, one per lane; their free entries' codes
+            const uint32_t nw = min(32u, gi.z - w0);
+            uint32_t x = 0;
+            if (row) {
+                if ((uint32_t)lane < nw) x = row[w0 + lane];
+            } else {
+                for (uint32_t k = 0; k < nw; ++k) {
+                    const uint32_t y = free_word(L, ow, geo.nw, (int)(w0 + k), lane);
+                    if ((uint32_t)lane == k) x = y;
+                }
+            }
+            uint32_t sc = __popc(x);
+            const uint32_t own = sc;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t o = __shfl_up_sync(0xffffffffu, sc, d);
+                if (lane >= d) sc += o;
+            }
+            const int nl = min((int)nw, __popc(__ballot_sync(0xffffffffu, sc <= (uint32_t)kFreeMax)));
+            if (lane < nl) {
+                uint16_t *at = wb.code + (sc - own);
+                for (; x; x &= x - 1u) *at++ = (uint16_t)(lane << 5 | (__ffs(x) - 1));
+            }
+            __syncwarp();
+            const int n = (int)__shfl_sync(0xffffffffu, sc, nl - 1);
+            for (int t0 = 0; t0 < n && !found; t0 += 32) {
                 u128 q = 0;
-                int a = -1, b = -1;
-                if (k < v.len) {
+                uint64_t mc = 0;
+                if (t0 + lane < n) {
                     real ratio, contrib;
-                    if (eval_entry<real, kC>(L, V, v, v.base + k, ratio, contrib, a, b)) q = rate_of<real>(ratio, &flag);
+                    if (flat_entry_value<real, kC>(L, V, single, w0 * 32u + wb.code[t0 + lane], ratio, contrib, mc))
+                        q = rate_of<real>(ratio, &flag);
                 }
                 const u128 incl2 = warp_incl_scan_u128(q, lane) + carry;
-                const unsigned hit = __ballot_sync(0xffffffffu, k < v.len && q != 0 && incl2 > Tl);
+                const unsigned hit = __ballot_sync(0xffffffffu, q != 0 && incl2 > Tl);
                 if (hit) {
-                    const int h = __ffs(hit) - 1;
-                    uint64_t c = 0;
-                    if (lane == h) {
-                        const uint64_t kind = v.kind == 0 ? 1 : 2;
-                        const uint64_t j10 = kind == 2 ? (uint64_t)v.j : 1023ull, b10 = kind == 2 ? (uint64_t)b : 1023ull;
-                        c = kind | ((uint64_t)v.i << 2) | (j10 << 12) | ((uint64_t)a << 22) | (b10 << 32);
-                    }
-                    code = __shfl_sync(0xffffffffu, c, h);
+                    code = __shfl_sync(0xffffffffu, mc, __ffs(hit) - 1);
                     found = true;
                 }
                 carry = shfl_u128(incl2, 31);
             }
+            __syncwarp();
+            w0 += (uint32_t)nl;
         }
         if (!found && lane == 0) atomicOr(status, VMC_DEV_INCONSISTENT);
     } else if (lane == 0) {
@@ -744,24 +1089,31 @@ __device__ __forceinline__ void select_walker(const ListsView &L, const WalkerAr
     }
 }
 
+// bits: the rows of all walkers, or null
 template <typename real, bool kC>
-__global__ void __launch_bounds__(512)
-k_ctmc_select(ListsView L, WalkerArgs A, CpsView C, const u128 *__restrict__ rates, uint64_t seed,
-              uint64_t *__restrict__ move_code, unsigned *status) {
-    const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+__global__ void __launch_bounds__(VMC_THREADS)
+k_ctmc_select(ListsView L, WalkerArgs A, CpsView C, const u128 *__restrict__ rates, const uint32_t *__restrict__ bits,
+              uint64_t seed, uint64_t *__restrict__ move_code, unsigned *status) {
+    __shared__ WarpBuf bufs[VMC_WARPS];
+    const int w = blockIdx.x * VMC_WARPS + (threadIdx.x >> 5);
     if (w >= A.W) return;
-    select_walker<real, kC>(L, A, w, rates, seed, move_code, status, C);
+    select_walker<real, kC>(L, A, w, rates, bits ? bits + (size_t)w * L.words : nullptr, seed, move_code, status,
+                            bufs[threadIdx.x >> 5], C);
 }
 
+// use_bits: the descriptors' rows hold all walkers (one round)
 template <typename real>
-__global__ void __launch_bounds__(512)
-k_ctmc_select_batched(const SysDesc *__restrict__ sys, int n_sys, int total, uint64_t seed, unsigned *status) {
-    const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+__global__ void __launch_bounds__(VMC_THREADS)
+k_ctmc_select_batched(const SysDesc *__restrict__ sys, int n_sys, int total, int use_bits, uint64_t seed, unsigned *status) {
+    __shared__ WarpBuf bufs[VMC_WARPS];
+    const int t = blockIdx.x * VMC_WARPS + (threadIdx.x >> 5);
     if (t >= total) return;
     int k = 0;
     while (k + 1 < n_sys && sys[k + 1].w_begin <= t) ++k;
     const SysDesc &d = sys[k];
-    select_walker<real, false>(d.L, d.A, t - d.w_begin, d.rates, seed, d.move_code, status);
+    const int w = t - d.w_begin;
+    select_walker<real, false>(d.L, d.A, w, d.rates, use_bits ? d.bits + (size_t)w * d.L.words : nullptr, seed, d.move_code,
+                               status, bufs[threadIdx.x >> 5]);
 }
 
 // Screened move set of one walker, written out in canonical order (Sec. II.A, II.B): one warp per
@@ -797,7 +1149,7 @@ k_screened_moves(ListsView L, WalkerArgs A, CpsView C, int w_begin, int n_w, int
             const int src = __ffs(mask) - 1;
             mask &= mask - 1;
             const Unit<real> v = shfl_unit(u, src);
-            if (v.base + v.len > list_size(L, v.kind)) {   // cannot happen: guard, never read
+            if (v.base + v.len > 32u * (uint32_t)L.words) {   // cannot happen: guard, never read
                 flag |= VMC_DEV_INCONSISTENT;
                 continue;
             }
@@ -846,7 +1198,7 @@ __device__ __forceinline__ void apply_walker(const ListsView &L, const WalkerArg
     if (code == 0) return;
     const int M = geo.M, ne = geo.ne, N2 = 2 * M;
     uint16_t *pos = (uint16_t *)smraw;
-    real *vec = (real *)(((uintptr_t)(pos + 2 * M) + 15) & ~(uintptr_t)15);
+    real *vec = (real *)(smraw + ((2 * sizeof(uint16_t) * (size_t)M + 15) & ~(size_t)15));
     // vec holds: ua[nmax], ub[nmax], gci[M], gcj[M], arow_i[nmax], arow_j[nmax]
     __shared__ double red[32];
     real *Gw = (real *)A.G + (size_t)w * geo.g_stride;
@@ -1099,8 +1451,27 @@ k_ctmc_apply_batched(const SysDesc *__restrict__ sys, int n_sys) {
 
 }  // namespace
 
-// per-warp entry queues of the local-energy kernel: 2 x 64 codes of 4 bytes
-static size_t eloc_queue_bytes(int threads) { return (size_t)(threads / 32) * 128 * sizeof(uint32_t); }
+// Shared memory of a local-energy CTA: G rows, orbital table, occupation words, warp buffers and the
+// correlator tables.
+static size_t eloc_smem_bytes(const ListsView &L, const vmc_walkers *Wk, const CpsView &C, int threads) {
+    const bool d = Wk->precision == VMC_FP64;
+    const size_t esz = d ? 8 : 4, M = (size_t)Wk->M, na = (size_t)Wk->n_alpha, nb = (size_t)Wk->n_beta;
+    const size_t g = esz * ((M - na) * (na + 1) + (M - nb) * (nb + 1)) + 8;
+    const size_t orb = (d ? OrbTable<double>::bytes : OrbTable<float>::bytes) * 2 * M + 4 * 2 * ((M + 31) / 32) + 16;
+    const size_t warps = (size_t)(threads / 32) * sizeof(WarpBuf);
+    // correlator product: 1/c per correlator (padded to 4), coefficient positions and offsets
+    const size_t cps = C.n_corr ? esz * (size_t)((C.n_corr + 3) & ~3) + 4 * (2 * (size_t)C.n_corr + 1) : 0;
+    const size_t own = own_rows(L.words, Wk->W) ? 4 * (size_t)L.words : 0;      // its bits
+    return g + orb + own + warps + cps;
+}
+
+// Which walkers the local energy takes: G rows, exp(S), orbital map, 512 bytes per warp and the correlator
+// tables (site lists included) within 200 KB (the CTA's own sum stays within the 227 KB that it can have).
+static bool eloc_fits(const vmc_walkers *Wk, const CpsView &C, int threads) {
+    const size_t esz = Wk->precision == VMC_FP64 ? 8 : 4, M = (size_t)Wk->M, na = (size_t)Wk->n_alpha, nb = (size_t)Wk->n_beta;
+    const size_t cps = C.n_corr ? esz * (size_t)((C.n_corr + 3) & ~3) + 4 * (2 * (size_t)C.n_corr + 1) + 4 * (M + 1) + 4 * (size_t)C.nnz : 0;
+    return esz * ((M - na) * (na + 1) + (M - nb) * (nb + 1) + 2 * M) + 4 * M + 16 + 512 * (size_t)(threads / 32) + cps <= 200 * 1024;
+}
 
 static WalkerArgs make_args(vmc_walkers *Wk) {
     WalkerArgs A;
@@ -1113,28 +1484,32 @@ static WalkerArgs make_args(vmc_walkers *Wk) {
     return A;
 }
 
-template <typename real, int kT>
-static cudaError_t eloc_launch_t(const vmc_ctx *ctx, int W, size_t smem, const ListsView &L, const WalkerArgs &A,
+template <typename real, int kT, bool kS>
+static cudaError_t eloc_launch_t(const vmc_ctx *ctx, int w0, int W, size_t smem, const ListsView &L, const WalkerArgs &A,
                                  const CpsView &C, double *e_loc, double *t_res, u128 *rates) {
+    const uint32_t *bits = own_rows(L.words, A.W) ? nullptr : (const uint32_t *)ctx->bits;
     cudaError_t e;
     if (C.n_corr) {
-        e = cudaFuncSetAttribute(k_local_energy_cps<real, kT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = cudaFuncSetAttribute(k_local_energy_cps<real, kT, kS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e == cudaSuccess)
-            k_local_energy_cps<real, kT><<<W, kT, smem, ctx->stream>>>(L, A, C, e_loc, t_res, rates, ctx->d_status);
+            e = launch_dependent(bits != nullptr, k_local_energy_cps<real, kT, kS>, dim3(W), kT, smem, ctx->stream, L, A, C,
+                                 w0, bits, e_loc, t_res, rates, ctx->d_status);
         return e;
     }
-    e = cudaFuncSetAttribute(k_local_energy<real, kT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) k_local_energy<real, kT><<<W, kT, smem, ctx->stream>>>(L, A, e_loc, t_res, rates, ctx->d_status);
+    e = cudaFuncSetAttribute(k_local_energy<real, kT, kS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess)
+        e = launch_dependent(bits != nullptr, k_local_energy<real, kT, kS>, dim3(W), kT, smem, ctx->stream, L, A, w0, bits,
+                             e_loc, t_res, rates, ctx->d_status);
     return e;
 }
-template <typename real>
-static cudaError_t eloc_launch(const vmc_ctx *ctx, int W, size_t smem, const ListsView &L, const WalkerArgs &A,
+template <typename real, bool kS>
+static cudaError_t eloc_launch(const vmc_ctx *ctx, int w0, int W, size_t smem, const ListsView &L, const WalkerArgs &A,
                                const CpsView &C, double *e_loc, double *t_res, u128 *rates) {
     switch (ctx->eloc_threads) {
-    case 128: return eloc_launch_t<real, 128>(ctx, W, smem, L, A, C, e_loc, t_res, rates);
-    case 256: return eloc_launch_t<real, 256>(ctx, W, smem, L, A, C, e_loc, t_res, rates);
-    case 384: return eloc_launch_t<real, 384>(ctx, W, smem, L, A, C, e_loc, t_res, rates);
-    default: return eloc_launch_t<real, 512>(ctx, W, smem, L, A, C, e_loc, t_res, rates);
+    case 128: return eloc_launch_t<real, 128, kS>(ctx, w0, W, smem, L, A, C, e_loc, t_res, rates);
+    case 256: return eloc_launch_t<real, 256, kS>(ctx, w0, W, smem, L, A, C, e_loc, t_res, rates);
+    case 384: return eloc_launch_t<real, 384, kS>(ctx, w0, W, smem, L, A, C, e_loc, t_res, rates);
+    default: return eloc_launch_t<real, 512, kS>(ctx, w0, W, smem, L, A, C, e_loc, t_res, rates);
     }
 }
 template <typename real, int kT>
@@ -1143,8 +1518,8 @@ static cudaError_t eloc_batched_launch_t(const vmc_ctx *ctx, int nsm, size_t se,
     cudaError_t e = cudaFuncSetAttribute(k_local_energy_batched<real, kT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)se);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_local_energy_batched<real, kT>, kT, se);
     if (e == cudaSuccess)
-        k_local_energy_batched<real, kT><<<std::max(1, per_sm) * nsm, kT, se, ctx->stream>>>(tab, n, total, ctx->d_queue,
-                                                                                            ctx->d_status);
+        e = launch_dependent(true, k_local_energy_batched<real, kT>, dim3(std::max(1, per_sm) * nsm), kT, se, ctx->stream, tab, n,
+                             total, ctx->d_queue, ctx->d_status);
     return e;
 }
 template <typename real>
@@ -1157,25 +1532,88 @@ static cudaError_t eloc_batched_launch(const vmc_ctx *ctx, int nsm, size_t se, c
     }
 }
 
+// Rate store and, behind it in the same allocation, the free-entry rows of one launch's walkers: at most
+// kBitsCap bytes of rows (but at least one tile of 32 walkers); a larger call runs in several launches of *chunk
+// walkers.  row = 0: no rows.  When the memory cannot be had the chunk is halved down to one tile.
+constexpr size_t kBitsCap = (size_t)1 << 30;
+
+static size_t row_bytes(const ListsView &L) { return std::max<size_t>(32, sizeof(uint32_t) * (size_t)L.words); }
+static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
+
+// Frees the store and allocates `bytes`; a failed allocation leaves none.
+static cudaError_t grow_store(vmc_ctx *ctx, size_t bytes) {
+    ctx->rates_valid = 0;
+    ctx->rates_batch.clear();
+    if (ctx->rates) {
+        const cudaError_t e = cudaStreamSynchronize(ctx->stream);
+        if (e != cudaSuccess) return e;
+        cudaFree(ctx->rates);
+        ctx->rates = nullptr;
+        ctx->rates_bytes = 0;
+    }
+    const cudaError_t e = cudaMalloc(&ctx->rates, bytes);
+    if (e == cudaSuccess) ctx->rates_bytes = bytes;
+    else ctx->rates = nullptr;
+    if (e == cudaErrorMemoryAllocation) cudaGetLastError();
+    return e;
+}
+
+static vmc_status ensure_store(vmc_ctx *ctx, size_t rates_bytes, size_t row, int W, int *chunk) {
+    const size_t r = align256(rates_bytes);
+    int n = row ? (W + 31) & ~31 : W;
+    if (row) {
+        const size_t fit = kBitsCap / row & ~(size_t)31;
+        if ((size_t)n > fit) n = std::max(32, (int)fit);
+    }
+    for (;; n = std::max(32, (n / 2 + 31) & ~31)) {
+        const size_t bytes = r + row * (size_t)n + 32;     // a read of two words may run past the last row
+        cudaError_t e = cudaSuccess;
+        if (bytes > ctx->rates_bytes) e = grow_store(ctx, bytes);
+        if (e == cudaSuccess) break;
+        if (e != cudaErrorMemoryAllocation || !row || n <= 32) return cuda_check(ctx, e, "rate store");
+    }
+    *chunk = n;
+    ctx->bits = (char *)ctx->rates + r;
+    return VMC_OK;
+}
+
+// Splits of a walker tile's row over CTAs: about 32 CTAs per SM (several short waves), each warp with at
+// least two pieces of 256 entries so that the tile's transposed occupations pay, or one while all
+// CTAs are resident at once (five per SM) and latency counts.
+static int free_bits_parts(int tiles, int words) {
+    const int pieces = words / 8, one = std::max(1, (pieces + 7) / 8);
+    if ((int64_t)one * tiles <= 152 * 5) return one;
+    const int want = (152 * 32 + tiles - 1) / tiles, most = std::max(1, (pieces + 15) / 16);
+    return std::max(1, std::min(want, most));
+}
+
 vmc_status launch_local_energy(vmc_ctx *ctx, const vmc_lists *L, vmc_walkers *Wk, const CpsView &C, double *e_loc,
-                               double *t_res, u128 *rates, int n_groups) {
-    const int M = Wk->M;
-    (void)n_groups;
-    const size_t esz = Wk->precision == VMC_FP64 ? 8 : 4;
-    const int na = Wk->n_alpha, nb = Wk->n_beta;
-    const size_t gpad = (size_t)(M - na) * (na + 1) + (size_t)(M - nb) * (nb + 1);
-    // correlator product: 1/c per correlator (padded to 4) and a 16-bit index per correlator
-    const size_t cps = C.n_corr ? esz * (size_t)((C.n_corr + 3) & ~3) + 4 * (2 * (size_t)C.n_corr + 1) +
-                                      4 * ((size_t)M + 1) + 4 * (size_t)C.nnz
-                                : 0;
-    const size_t smem = esz * (gpad + 2 * (size_t)M) + 2 * (2 * (size_t)M) + 16 + eloc_queue_bytes(ctx->eloc_threads) + cps;
-    if (smem > 200 * 1024) return set_err(ctx, VMC_ERR_ARG, "walker G table does not fit in shared memory");
+                               double *t_res) {
+    const size_t smem = eloc_smem_bytes(L->view, Wk, C, ctx->eloc_threads);
+    if (!eloc_fits(Wk, C, ctx->eloc_threads)) return set_err(ctx, VMC_ERR_ARG, "walker G table does not fit in shared memory");
     WalkerArgs A = make_args(Wk);
-    cudaError_t e = Wk->precision == VMC_FP64
-                              ? eloc_launch<double>(ctx, Wk->W, smem, L->view, A, C, e_loc, t_res, rates)
-                              : eloc_launch<float>(ctx, Wk->W, smem, L->view, A, C, e_loc, t_res, rates);
-    ctx->launches += 1;
-    if (e == cudaSuccess) e = cudaGetLastError();
+    const bool own = own_rows(L->view.words, Wk->W);
+    ctx->bits_whole = 0;
+    int chunk = Wk->W;
+    const size_t rates_bytes = sizeof(u128) * rate_store_units(Wk->W, L->view.n_groups);
+    vmc_status st = ensure_store(ctx, rates_bytes, own ? 0 : row_bytes(L->view), Wk->W, &chunk);
+    if (st) return st;
+    u128 *rates = (u128 *)ctx->rates;
+    cudaError_t e = cudaSuccess;
+    for (int w0 = 0; w0 < Wk->W && e == cudaSuccess; w0 += chunk) {
+        const int n = std::min(chunk, Wk->W - w0), tiles = (n + kTile - 1) / kTile;
+        if (!own) {
+            k_free_bits<<<dim3(tiles, free_bits_parts(tiles, L->view.words)), 256, 0, ctx->stream>>>(
+                L->view, A.occ_bits, w0, w0 + n, (uint32_t *)ctx->bits);
+            ctx->launches += 1;
+        }
+        if (Wk->precision != VMC_FP64) e = eloc_launch<float, false>(ctx, w0, n, smem, L->view, A, C, e_loc, t_res, rates);
+        else if (L->view.scaled) e = eloc_launch<double, true>(ctx, w0, n, smem, L->view, A, C, e_loc, t_res, rates);
+        else e = eloc_launch<double, false>(ctx, w0, n, smem, L->view, A, C, e_loc, t_res, rates);
+        ctx->launches += 1;
+        if (e == cudaSuccess) e = cudaGetLastError();
+    }
+    ctx->bits_whole = !own && chunk >= Wk->W;      // for the choice of the next move
     return cuda_check(ctx, e, "k_local_energy");
 }
 
@@ -1184,7 +1622,8 @@ static cudaError_t ctmc_launch(vmc_ctx *ctx, const vmc_lists *L, const vmc_param
                                const CpsView &C, int W, size_t smem, uint64_t seed, const u128 *rates,
                                uint64_t *move_code) {
     const int sel_blocks = (W + VMC_WARPS - 1) / VMC_WARPS;
-    k_ctmc_select<real, kC><<<sel_blocks, VMC_THREADS, 0, ctx->stream>>>(L->view, A, C, rates, seed, move_code,
+    const uint32_t *bits = ctx->bits_whole ? (const uint32_t *)ctx->bits : nullptr;
+    k_ctmc_select<real, kC><<<sel_blocks, VMC_THREADS, 0, ctx->stream>>>(L->view, A, C, rates, bits, seed, move_code,
                                                                          ctx->d_status);
     cudaError_t e = cudaFuncSetAttribute(k_ctmc_apply<real, kC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) k_ctmc_apply<real, kC><<<W, VMC_THREADS, smem, ctx->stream>>>(L->view, A, C, P->J, move_code);
@@ -1213,24 +1652,27 @@ vmc_status launch_ctmc_step(vmc_ctx *ctx, const vmc_lists *L, const vmc_params *
 }
 
 // ---------------------------------------------------------------------------------- batches
-static size_t eloc_smem_bytes(const vmc_lists *L, const vmc_walkers *Wk, int threads) {
-    const size_t esz = Wk->precision == VMC_FP64 ? 8 : 4;
-    const int M = Wk->M, na = Wk->n_alpha, nb = Wk->n_beta;
-    const size_t gpad = (size_t)(M - na) * (na + 1) + (size_t)(M - nb) * (nb + 1);
-    (void)L;
-    return esz * (gpad + 2 * (size_t)M) + 2 * (2 * (size_t)M) + 16 + eloc_queue_bytes(threads);
-}
-
 static size_t apply_smem_bytes(const vmc_walkers *Wk) {
     const int M = Wk->M, nmax = Wk->n_alpha > Wk->n_beta ? Wk->n_alpha : Wk->n_beta;
     const size_t esz = Wk->precision == VMC_FP64 ? 8 : 4;
     return 2 * (2 * (size_t)M) + 32 + esz * (4 * (size_t)((nmax + 3) & ~3) + 2 * (size_t)((M + 3) & ~3));
 }
 
-// Builds (and uploads when changed) the descriptor table of a batch, most expensive systems
-// first.  Also sizes the shared rate store.  Outputs: total walkers, max shared memory.
-static vmc_status prepare_batch(vmc_ctx *ctx, int n, const vmc_batch_item *items, int *total,
-                                size_t *smem_eloc, size_t *smem_apply, int *precision) {
+// A batch as launched: walkers, shared memory, rounds of the local energy and, per round, the walkers
+// and walker tiles.
+struct BatchPlan {
+    int total = 0, precision = 0, rounds = 1;
+    bool fits = true;                  // every system's walkers fit the local energy's shared memory
+    size_t smem_eloc = 0, smem_apply = 0;
+    std::vector<int> walkers, tiles;   // per round
+    int words = 0;                     // the longest free-entry row
+};
+
+// Builds (and uploads when changed) the descriptor tables of a batch, most expensive systems first:
+// one table over all walkers (used by the CTMC step, and by the local energy when one round is enough),
+// then one per round of the local energy.  Also sizes the shared rate store and the free-entry rows:
+// every system's walkers are split over as few rounds as keep the rows within kBitsCap.
+static vmc_status prepare_batch(vmc_ctx *ctx, int n, const vmc_batch_item *items, BatchPlan &plan) {
     extern vmc_status lists_set_eps(vmc_ctx *, vmc_lists *, double);
     if (n < 1 || n > 64 || !items) return set_err(ctx, VMC_ERR_ARG, "1 to 64 batch items");
     std::vector<int> order(n);
@@ -1260,20 +1702,44 @@ static vmc_status prepare_batch(vmc_ctx *ctx, int n, const vmc_batch_item *items
         rate_off[k] = rates_total;
         rates_total += rate_store_units(it.walkers->W, it.lists->view.n_groups);
         tot += it.walkers->W;
-        se = std::max(se, eloc_smem_bytes(it.lists, it.walkers, ctx->eloc_threads));
+        se = std::max(se, eloc_smem_bytes(it.lists->view, it.walkers, CpsView{}, ctx->eloc_threads));
+        plan.fits = plan.fits && eloc_fits(it.walkers, CpsView{}, ctx->eloc_threads);
         sa = std::max(sa, apply_smem_bytes(it.walkers));
     }
-    if (rates_total * sizeof(u128) > ctx->rates_bytes) {
-        if (ctx->rates) { cudaStreamSynchronize(ctx->stream); cudaFree(ctx->rates); ctx->rates = nullptr; }
-        cudaError_t e = cudaMalloc(&ctx->rates, rates_total * sizeof(u128));
-        if (e != cudaSuccess) { ctx->rates_bytes = 0; return cuda_check(ctx, e, "batched rate store"); }
-        ctx->rates_bytes = rates_total * sizeof(u128);
+    // free-entry rows: rounds (doubled) until every system's share fits
+    const size_t bits_at = align256(rates_total * sizeof(u128));
+    std::vector<int> share(n);
+    int rounds = 1;
+    for (;; rounds *= 2) {
+        size_t bytes = bits_at + 32;
+        bool more = false;
+        for (int k = 0; k < n; ++k) {
+            const vmc_batch_item &it = items[order[k]];
+            share[k] = ((it.walkers->W + rounds - 1) / rounds + 31) & ~31;
+            more = more || share[k] > 32;
+            bytes += row_bytes(it.lists->view) * (size_t)share[k];
+        }
+        if (bytes <= ctx->rates_bytes) break;
+        if (bytes - bits_at > kBitsCap && more) continue;
+        const cudaError_t e = grow_store(ctx, bytes);
+        if (e == cudaSuccess) break;
+        if (e != cudaErrorMemoryAllocation || !more) return cuda_check(ctx, e, "batched rate store");
     }
-    std::string tab(sizeof(SysDesc) * n, '\0');
+    plan.rounds = rounds;
+    const int n_tabs = rounds == 1 ? 1 : rounds + 1;
+    std::string tab(sizeof(SysDesc) * n * n_tabs, '\0');
     SysDesc *d = (SysDesc *)&tab[0];
-    int wb = 0;
+    int wb = 0, tb = 0;
+    size_t bit_off = bits_at;
     for (int k = 0; k < n; ++k) {
         const vmc_batch_item &it = items[order[k]];
+        plan.words = std::max(plan.words, it.lists->view.words);
+        d[k].bits = (uint32_t *)((char *)ctx->rates + bit_off);
+        bit_off += row_bytes(it.lists->view) * (size_t)share[k];
+        d[k].w_first = 0;
+        d[k].w_count = it.walkers->W;
+        d[k].t_begin = tb;
+        tb += (it.walkers->W + kTile - 1) / kTile;
         d[k].L = it.lists->view;
         d[k].A = make_args(it.walkers);
         d[k].J = it.params->J;
@@ -1283,6 +1749,22 @@ static vmc_status prepare_batch(vmc_ctx *ctx, int n, const vmc_batch_item *items
         d[k].move_code = it.d_move_code;
         d[k].w_begin = wb;
         wb += it.walkers->W;
+    }
+    if (rounds == 1) { plan.walkers.push_back(wb); plan.tiles.push_back(tb); }
+    for (int r = 0; rounds > 1 && r < rounds; ++r) {
+        int w = 0, t = 0;
+        for (int k = 0; k < n; ++k) {
+            SysDesc &x = d[(size_t)(r + 1) * n + k];
+            x = d[k];
+            x.w_first = std::min(r * share[k], d[k].w_count);
+            x.w_count = std::min(share[k], d[k].w_count - x.w_first);
+            x.w_begin = w;
+            x.t_begin = t;
+            w += x.w_count;
+            t += (x.w_count + kTile - 1) / kTile;
+        }
+        plan.walkers.push_back(w);
+        plan.tiles.push_back(t);
     }
     if (tab != ctx->batch_host) {
         if (tab.size() > ctx->batch_desc_bytes) {
@@ -1300,10 +1782,10 @@ static vmc_status prepare_batch(vmc_ctx *ctx, int n, const vmc_batch_item *items
         if (e != cudaSuccess) return cuda_check(ctx, e, "batch table upload");
         ctx->batch_host = tab;
     }
-    *total = tot;
-    *smem_eloc = se;
-    *smem_apply = sa;
-    *precision = items[0].walkers->precision;
+    plan.total = tot;
+    plan.smem_eloc = se;
+    plan.smem_apply = sa;
+    plan.precision = items[0].walkers->precision;
     return VMC_OK;
 }
 
@@ -1314,21 +1796,26 @@ static std::string batch_signature(int n, const vmc_batch_item *items) {
 }
 
 vmc_status launch_local_energy_batch(vmc_ctx *ctx, int n, const vmc_batch_item *items) {
-    int total = 0, prec = 0;
-    size_t se = 0, sa = 0;
-    vmc_status st = prepare_batch(ctx, n, items, &total, &se, &sa, &prec);
+    BatchPlan plan;
+    vmc_status st = prepare_batch(ctx, n, items, plan);
     if (st) return st;
-    if (se > 200 * 1024) return set_err(ctx, VMC_ERR_ARG, "walker G table does not fit in shared memory");
-    cudaError_t e = cudaMemsetAsync(ctx->d_queue, 0, sizeof(int), ctx->stream);
+    const size_t se = plan.smem_eloc;
+    if (!plan.fits) return set_err(ctx, VMC_ERR_ARG, "walker G table does not fit in shared memory");
     int dev = 0, nsm = 0;
-    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const SysDesc *tab = (const SysDesc *)ctx->batch_desc;
-    if (e == cudaSuccess)
-        e = prec == VMC_FP64 ? eloc_batched_launch<double>(ctx, nsm, se, tab, n, total)
-                             : eloc_batched_launch<float>(ctx, nsm, se, tab, n, total);
-    ctx->launches += 1;
-    if (e == cudaSuccess) e = cudaGetLastError();
+    for (int r = 0; r < plan.rounds && e == cudaSuccess; ++r) {
+        const SysDesc *tab = (const SysDesc *)ctx->batch_desc + (plan.rounds > 1 ? (size_t)(r + 1) * n : 0);
+        const int total = plan.walkers[r], tiles = plan.tiles[r];
+        if (!total) continue;
+        e = cudaMemsetAsync(ctx->d_queue, 0, sizeof(int), ctx->stream);
+        if (e != cudaSuccess) break;
+        k_free_bits_batched<<<dim3(tiles, free_bits_parts(tiles, plan.words)), 256, 0, ctx->stream>>>(tab, n);
+        e = plan.precision == VMC_FP64 ? eloc_batched_launch<double>(ctx, nsm, se, tab, n, total)
+                                       : eloc_batched_launch<float>(ctx, nsm, se, tab, n, total);
+        ctx->launches += 2;
+        if (e == cudaSuccess) e = cudaGetLastError();
+    }
     if (e != cudaSuccess) return cuda_check(ctx, e, "k_local_energy_batched");
     ctx->rates_batch = batch_signature(n, items);
     ctx->rates_valid = 0;
@@ -1338,19 +1825,22 @@ vmc_status launch_local_energy_batch(vmc_ctx *ctx, int n, const vmc_batch_item *
 vmc_status launch_ctmc_step_batch(vmc_ctx *ctx, int n, const vmc_batch_item *items, uint64_t seed) {
     if (ctx->rates_batch.empty() || ctx->rates_batch != batch_signature(n, items))
         return set_err(ctx, VMC_ERR_ARG, "vmc_local_energy_batch must precede vmc_ctmc_step_batch on the same items");
-    int total = 0, prec = 0;
-    size_t se = 0, sa = 0;
-    vmc_status st = prepare_batch(ctx, n, items, &total, &se, &sa, &prec);
+    BatchPlan plan;
+    vmc_status st = prepare_batch(ctx, n, items, plan);
     if (st) return st;
+    const int total = plan.total, prec = plan.precision;
+    const size_t sa = plan.smem_apply;
     const SysDesc *tab = (const SysDesc *)ctx->batch_desc;
-    const int sel_blocks = (total + 7) / 8;
+    const int sel_blocks = (total + VMC_WARPS - 1) / VMC_WARPS, use_bits = plan.rounds == 1 ? 1 : 0;
     cudaError_t e;
     if (prec == VMC_FP64) {
-        k_ctmc_select_batched<double><<<sel_blocks, 256, 0, ctx->stream>>>(tab, n, total, seed, ctx->d_status);
+        k_ctmc_select_batched<double><<<sel_blocks, VMC_THREADS, 0, ctx->stream>>>(tab, n, total, use_bits, seed,
+                                                                                ctx->d_status);
         e = cudaFuncSetAttribute(k_ctmc_apply_batched<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sa);
         if (e == cudaSuccess) k_ctmc_apply_batched<double><<<total, 256, sa, ctx->stream>>>(tab, n);
     } else {
-        k_ctmc_select_batched<float><<<sel_blocks, 256, 0, ctx->stream>>>(tab, n, total, seed, ctx->d_status);
+        k_ctmc_select_batched<float><<<sel_blocks, VMC_THREADS, 0, ctx->stream>>>(tab, n, total, use_bits, seed,
+                                                                                ctx->d_status);
         e = cudaFuncSetAttribute(k_ctmc_apply_batched<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sa);
         if (e == cudaSuccess) k_ctmc_apply_batched<float><<<total, 256, sa, ctx->stream>>>(tab, n);
     }

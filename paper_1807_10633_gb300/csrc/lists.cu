@@ -244,80 +244,137 @@ const char *check_build_args(int M, const double *h1, const double *eri, int eri
 // (p, p + band] followed by the opposite-spin q in [p - band, p + band]; then beta rows, rpg of them
 // per group (lane = row offset x band + candidate) or cpr_b chunks each.  Groups and lanes run in
 // ascending (i, j) order, which is the canonical order of the CTMC choice.
-static void build_unit_table(const vmc_lists *L, const uint32_t *s_len, const uint32_t *ds_len,
-                             const uint32_t *do_len, std::vector<uint4> &tab) {
-    const ListsView &v = L->view;
-    const int M = L->M, Gs = (2 * M + 31) / 32;
-    tab.assign((size_t)v.n_groups * 32, make_uint4(0, 0, 0, 0));
-    auto ncand = [&](int i) {   // candidates of spin-orbital row i
-        const int sp = i >= M, p = i - sp * M, nS = std::min(v.band, M - 1 - p);
-        return sp ? nS : nS + (std::min(M - 1, p + v.band) - std::max(0, p - v.band) + 1);
-    };
-    auto cand = [&](int i, int t) {
-        const int sp = i >= M, p = i - sp * M, nS = std::min(v.band, M - 1 - p);
-        return t < nS ? i + 1 + t : M + std::max(0, p - v.band) + (t - nS);
-    };
-    for (int g = 0; g < v.n_groups; ++g)
-        for (int lane = 0; lane < 32; ++lane) {
-            uint4 &e = tab[(size_t)g * 32 + lane];
-            if (g < Gs) {
-                const int i = g * 32 + lane;
-                if (i >= 2 * M) continue;
-                const int sp = i >= M, p = i - sp * M;
-                e = make_uint4((uint32_t)p, L->h_s_off[p], s_len[p], (uint32_t)(sp << 2));
-                continue;
-            }
-            const int ga = g - Gs;
-            int i, t;
-            if (ga < M * v.cpr) {
-                i = ga / v.cpr;
-                t = (ga % v.cpr) * 32 + lane;
-            } else if (v.rpg > 1) {
-                const int ro = lane / v.band;
-                i = M + (ga - M * v.cpr) * v.rpg + ro;
-                t = lane - ro * v.band;
-                if (ro >= v.rpg || i >= 2 * M) continue;
-            } else {
-                const int gb = ga - M * v.cpr;
-                i = M + gb / v.cpr_b;
-                t = (gb % v.cpr_b) * 32 + lane;
-            }
-            if (t >= ncand(i)) continue;
-            const int j = cand(i, t);
-            const int si = i >= M, sj = j >= M, pi = i - si * M, pj = j - sj * M;
-            if (si == sj) {
-                const int tt = tri_index(pi, pj, M);
-                e = make_uint4((uint32_t)pi | ((uint32_t)pj << 16), L->h_ds_off[tt], ds_len[tt], (uint32_t)(1 | (si << 2)));
-            } else {
-                const int tt = pi * M + pj;
-                e = make_uint4((uint32_t)pi | ((uint32_t)pj << 16), L->h_do_off[tt], do_len[tt], 2u);
-            }
-        }
+struct UnitId {
+    int kind, spin;    // 0 single, 1 same-spin double, 2 opposite-spin double; spin of kinds 0 and 1
+    int p, q, list;    // spatial orbitals of i and j (q = p for singles); index of its list in its class
+};
+
+static bool unit_of(const ListsView &v, int g, int lane, UnitId &u) {
+    const int M = v.M, Gs = (2 * M + 31) / 32;
+    if (g < Gs) {
+        const int i = g * 32 + lane;
+        if (i >= 2 * M) return false;
+        u.kind = 0;
+        u.spin = i >= M;
+        u.p = u.q = u.list = i - u.spin * M;
+        return true;
+    }
+    const int ga = g - Gs;
+    int i, t;
+    if (ga < M * v.cpr) {
+        i = ga / v.cpr;
+        t = (ga % v.cpr) * 32 + lane;
+    } else if (v.rpg > 1) {
+        const int ro = lane / v.band;
+        i = M + (ga - M * v.cpr) * v.rpg + ro;
+        t = lane - ro * v.band;
+        if (ro >= v.rpg || i >= 2 * M) return false;
+    } else {
+        const int gb = ga - M * v.cpr;
+        i = M + gb / v.cpr_b;
+        t = (gb % v.cpr_b) * 32 + lane;
+    }
+    const int sp = i >= M, p = i - sp * M, nS = std::min(v.band, M - 1 - p), lo = std::max(0, p - v.band);
+    const int n_cand = sp ? nS : nS + (std::min(M - 1, p + v.band) - lo + 1);   // candidates of row i
+    if (t >= n_cand) return false;
+    u.p = p;
+    if (t < nS) {
+        u.kind = 1;
+        u.spin = sp;
+        u.q = p + 1 + t;
+        u.list = tri_index(p, u.q, M);
+    } else {
+        u.kind = 2;
+        u.spin = 0;
+        u.q = lo + (t - nS);
+        u.list = p * M + u.q;
+    }
+    return true;
 }
 
-// Effective list lengths for eps_run (host binary searches, one small upload) and the unit table.
+// The flat entries (see ListsView) of host lists, with Jastrow constants 1.
+struct FlatLists {
+    std::vector<uint32_t> key, base;
+    std::vector<uint8_t> wcls;
+    std::vector<float4> r32;
+    std::vector<double4_32a> r64;
+    std::vector<uint4> group;
+};
+
+static void build_flat(const ListsView &v, const HostLists &H, FlatLists &F) {
+    auto bits_d = [](uint32_t u) { double d = 0.0; uint64_t x = u; memcpy(&d, &x, 8); return d; };
+    auto bits_f = [](uint32_t u) { float f; memcpy(&f, &u, 4); return f; };
+    auto align = [&](size_t to, uint8_t cls) {     // fill up to a multiple of `to` entries
+        while (F.key.size() % to) {
+            if (F.key.size() % 32 == 0) F.wcls.push_back(cls);
+            F.key.push_back(0);
+            F.r32.push_back(make_float4(0.f, 0.f, 0.f, 0.f));
+            F.r64.push_back(make_double4_32a(0.0, 0.0, 0.0, 0.0));
+        }
+    };
+    F.base.assign((size_t)v.n_groups * 32, 0);
+    for (int g = 0; g < v.n_groups; ++g) {
+        align(64, 0);
+        uint4 info = make_uint4((uint32_t)(F.key.size() / 32), 0xFFFFFFFFu, 0, 0);
+        int last = -1;
+        for (int lane = 0; lane < 32; ++lane) {
+            UnitId u;
+            if (!unit_of(v, g, lane, u)) continue;
+            const uint8_t cls = u.kind == 2 ? 2 : (u.spin ? 3 : 0);
+            if (last >= 0 && cls != last) align(32, (uint8_t)last);
+            last = cls;
+            if (u.kind == 1) {
+                const int ui = u.spin && v.rpg > 1 ? v.band - 1 : 0;
+                info.w = (info.w & ~0x7FFu) | (uint32_t)u.spin | (uint32_t)(ui & 31) << 1 |
+                         (uint32_t)((lane - u.q - u.p * ui) & 31) << 6;
+            }
+            if (u.kind == 2) info.w = (info.w & 0x7FFu) | (uint32_t)((lane - u.q) & 31) << 11;
+            if (u.kind == 2 && info.y == 0xFFFFFFFFu) info.y = (uint32_t)(F.key.size() / 32);
+            F.base[(size_t)g * 32 + lane] = (uint32_t)F.key.size();
+            const uint32_t *off = u.kind == 0 ? H.s_off.data() : (u.kind == 1 ? H.ds_off.data() : H.do_off.data());
+            for (uint32_t e = off[u.list]; e < off[u.list + 1]; ++e) {
+                const uint32_t ab = u.kind == 0 ? (uint32_t)H.s_a[e] | ((uint32_t)H.s_a[e] << 16)
+                                                : (u.kind == 1 ? H.ds_ab[e] : H.do_ab[e]);
+                const double x = u.kind == 0 ? 0.0 : (u.kind == 1 ? H.ds_v[e] : H.do_v[e]);
+                const uint32_t key = (ab & 0xFFu) | ((ab >> 16 & 0xFFu) << 8) | ((uint32_t)u.p << 16) | ((uint32_t)u.q << 24);
+                const uint32_t aux = u.kind == 0 ? (uint32_t)(u.spin * H.ns_pad) + e : 0u;
+                if (F.key.size() % 32 == 0) F.wcls.push_back(cls);
+                F.key.push_back(key);
+                F.r32.push_back(make_float4(bits_f(key), (float)x, 1.0f, bits_f(aux)));
+                F.r64.push_back(make_double4_32a(bits_d(key), x, 1.0, bits_d(aux)));
+            }
+        }
+        align(32, (uint8_t)std::max(0, last));
+        info.z = (uint32_t)(F.key.size() / 32);
+        if (info.y == 0xFFFFFFFFu) info.y = info.z;
+        F.group.push_back(info);
+    }
+    align(256, 0);
+}
+
+// Effective list lengths for eps_run (host binary searches): the unit table and the alive bits.
 vmc_status lists_set_eps(vmc_ctx *ctx, vmc_lists *L, double eps_run) {
     if (L->eps_run == eps_run) return VMC_OK;
-    const int M = L->M;
-    const int npair = M * (M - 1) / 2;
-    std::vector<uint32_t> s_len(M), ds_len(npair > 0 ? npair : 1), do_len((size_t)M * M);
-    for (int i = 0; i < M; ++i)
-        s_len[i] = count_above(L->h_s_key + L->h_s_off[i], L->h_s_off[i + 1] - L->h_s_off[i], eps_run);
-    for (int t = 0; t < npair; ++t)
-        ds_len[t] = count_above(L->h_ds_key + L->h_ds_off[t], L->h_ds_off[t + 1] - L->h_ds_off[t], eps_run);
-    for (int t = 0; t < M * M; ++t)
-        do_len[t] = count_above(L->h_do_key + L->h_do_off[t], L->h_do_off[t + 1] - L->h_do_off[t], eps_run);
-    std::vector<uint4> tab;
-    build_unit_table(L, s_len.data(), ds_len.data(), do_len.data(), tab);
+    const ListsView &v = L->view;
+    std::vector<uint4> tab((size_t)v.n_groups * 32, make_uint4(0, 0, 0, 0));
+    std::vector<uint32_t> alive((size_t)v.words + 1, 0u);
+    for (int g = 0; g < v.n_groups; ++g)
+        for (int lane = 0; lane < 32; ++lane) {
+            UnitId u;
+            if (!unit_of(v, g, lane, u)) continue;
+            const uint32_t *off = u.kind == 0 ? L->h_s_off : (u.kind == 1 ? L->h_ds_off : L->h_do_off);
+            const double *key = u.kind == 0 ? L->h_s_key : (u.kind == 1 ? L->h_ds_key : L->h_do_key);
+            const uint32_t n = count_above(key + off[u.list], off[u.list + 1] - off[u.list], eps_run);
+            const uint32_t base = L->h_base[(size_t)g * 32 + lane];
+            tab[(size_t)g * 32 + lane] = make_uint4((uint32_t)u.p | ((uint32_t)(u.kind == 0 ? 0 : u.q) << 16), base, n,
+                                                    (uint32_t)(u.kind | (u.spin << 2)));
+            for (uint32_t e = base; e < base + n; ++e) alive[e >> 5] |= 1u << (e & 31u);
+        }
     cudaError_t e;
-    e = cudaMemcpyAsync((void *)L->view.unit_tab, tab.data(), sizeof(uint4) * tab.size(), cudaMemcpyHostToDevice,
-                        ctx->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync((void *)L->view.s_len, s_len.data(), sizeof(uint32_t) * M, cudaMemcpyHostToDevice, ctx->stream);
-    if (e == cudaSuccess && npair > 0)
-        e = cudaMemcpyAsync((void *)L->view.ds_len, ds_len.data(), sizeof(uint32_t) * npair, cudaMemcpyHostToDevice, ctx->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync((void *)L->view.do_len, do_len.data(), sizeof(uint32_t) * M * M, cudaMemcpyHostToDevice, ctx->stream);
+    e = cudaMemcpyAsync((void *)v.unit_tab, tab.data(), sizeof(uint4) * tab.size(), cudaMemcpyHostToDevice, ctx->stream);
+    if (e == cudaSuccess && v.words > 0)
+        e = cudaMemcpyAsync((void *)v.alive, alive.data(), sizeof(uint32_t) * (size_t)v.words, cudaMemcpyHostToDevice,
+                            ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);   // host vectors go out of scope
     if (e != cudaSuccess) return cuda_check(ctx, e, "uploading list lengths");
     L->eps_run = eps_run;
@@ -347,7 +404,6 @@ extern "C" vmc_status vmc_build_screened_lists(vmc_ctx *ctx, int M, const double
     if (const char *why = check_build_args(M, h1, eri, eri_packed, eps)) return set_err(ctx, VMC_ERR_ARG, why);
     *out = nullptr;
     const size_t MM = (size_t)M;
-    const int npair = M * (M - 1) / 2;
     HostLists H;
     build_host(M, h1, Eri{eri, MM, eri_packed}, eps, H);
     const int64_t ns = H.ns, nds = H.nds, ndo = H.ndo, ns_pad = H.ns_pad;
@@ -372,30 +428,13 @@ extern "C" vmc_status vmc_build_screened_lists(vmc_ctx *ctx, int M, const double
     L->h_s_off = dup_u32(H.s_off); L->h_ds_off = dup_u32(H.ds_off); L->h_do_off = dup_u32(H.do_off);
     L->h_s_key = dup_f64(H.s_key); L->h_ds_key = dup_f64(H.ds_key); L->h_do_key = dup_f64(H.do_key);
 
-    // packed per-entry records (the Jastrow constants are rewritten by every refresh)
-    std::vector<float4> s_r32(ns + 1), ds_r32(nds + 1), do_r32(ndo + 1);
-    std::vector<double4_32a> s_r64(ns + 1), ds_r64(nds + 1), do_r64(ndo + 1);
-    auto bits_d = [](uint32_t u) { double d = 0.0; uint64_t x = u; memcpy(&d, &x, 8); return d; };
-    auto bits_f = [](uint32_t u) { float f; memcpy(&f, &u, 4); return f; };
-    for (int64_t e = 0; e < ns; ++e) {
-        s_r32[e] = make_float4(bits_f(H.s_a[e]), 1.0f, 1.0f, 0.0f);
-        s_r64[e] = make_double4_32a(bits_d(H.s_a[e]), 1.0, 1.0, 0.0);
-    }
-    for (int64_t e = 0; e < nds; ++e) {
-        ds_r32[e] = make_float4(bits_f(H.ds_ab[e]), (float)H.ds_v[e], 1.0f, 1.0f);
-        ds_r64[e] = make_double4_32a(bits_d(H.ds_ab[e]), H.ds_v[e], 1.0, 1.0);
-    }
-    for (int64_t e = 0; e < ndo; ++e) {
-        do_r32[e] = make_float4(bits_f(H.do_ab[e]), (float)H.do_v[e], 1.0f, 0.0f);
-        do_r64[e] = make_double4_32a(bits_d(H.do_ab[e]), H.do_v[e], 1.0, 0.0);
-    }
     std::vector<float> Tjf(MM * (ns_pad + 1)), Tjkf(MM * (ns_pad + 1));
     for (size_t k = 0; k < Tjf.size(); ++k) {
         Tjf[k] = (float)H.Tj[k];
         Tjkf[k] = (float)H.Tjk[k];
     }
 
-    // ---- work-unit geometry (see build_unit_table)
+    // ---- work-unit geometry (see unit_of)
     ListsView &v = L->view;
     v.M = M; v.ns = ns; v.nds = nds; v.ndo = ndo; v.e_core = e_core; v.ns_pad = ns_pad;
     {
@@ -413,6 +452,19 @@ extern "C" vmc_status vmc_build_screened_lists(vmc_ctx *ctx, int M, const double
         v.n_groups = (2 * M + 31) / 32 + M * v.cpr + nb_groups;
     }
 
+    FlatLists F;
+    build_flat(v, H, F);
+    if (F.key.size() >= (size_t)1 << 32) {
+        vmc_lists_destroy(L);
+        return set_err(ctx, VMC_ERR_ARG, "more than 2^32 list entries");
+    }
+    v.words = (int)(F.key.size() / 32);
+    L->h_base = dup_u32(F.base);
+    // scaling costs two products for each of about M^2 / 2 elements of G and saves four per free double; about
+    // one entry in eight is free.  (8 x 8 Hubbard lattice, singles alone: 68 us without, 86 us with it for
+    // 4,000 walkers; H160 at 1e-6: 13.2 -> 11.5 ms with it for 32,768.)
+    v.scaled = F.key.size() >= 2 * MM * MM ? 1 : 0;
+
     // ---- one device allocation
     struct Piece { const void *src; size_t bytes; size_t off; };
     std::vector<Piece> pcs;
@@ -422,24 +474,14 @@ extern "C" vmc_status vmc_build_screened_lists(vmc_ctx *ctx, int M, const double
         off = align256(off + (bytes ? bytes : 1));
         return pcs.size() - 1;
     };
-    const size_t i_s_off = add(H.s_off.data(), sizeof(uint32_t) * (M + 1));
-    const size_t i_s_len = add(nullptr, sizeof(uint32_t) * M);
     const size_t i_s_owner = add(H.s_owner.data(), sizeof(uint32_t) * ns);
     const size_t i_s_a = add(H.s_a.data(), sizeof(uint16_t) * ns);
-    const size_t i_s_r32 = add(s_r32.data(), sizeof(float4) * ns);
-    const size_t i_s_r64 = add(s_r64.data(), sizeof(double4_32a) * ns);
-    const size_t i_ds_off = add(H.ds_off.data(), sizeof(uint32_t) * (npair + 1));
-    const size_t i_ds_len = add(nullptr, sizeof(uint32_t) * (npair > 0 ? npair : 1));
-    const size_t i_ds_ab = add(H.ds_ab.data(), sizeof(uint32_t) * nds);
-    const size_t i_ds_owner = add(H.ds_owner.data(), sizeof(uint32_t) * nds);
-    const size_t i_ds_r32 = add(ds_r32.data(), sizeof(float4) * nds);
-    const size_t i_ds_r64 = add(ds_r64.data(), sizeof(double4_32a) * nds);
-    const size_t i_do_off = add(H.do_off.data(), sizeof(uint32_t) * (MM * MM + 1));
-    const size_t i_do_len = add(nullptr, sizeof(uint32_t) * MM * MM);
-    const size_t i_do_ab = add(H.do_ab.data(), sizeof(uint32_t) * ndo);
-    const size_t i_do_owner = add(H.do_owner.data(), sizeof(uint32_t) * ndo);
-    const size_t i_do_r32 = add(do_r32.data(), sizeof(float4) * ndo);
-    const size_t i_do_r64 = add(do_r64.data(), sizeof(double4_32a) * ndo);
+    const size_t i_key = add(F.key.data(), sizeof(uint32_t) * F.key.size());
+    const size_t i_alive = add(nullptr, sizeof(uint32_t) * (size_t)v.words);
+    const size_t i_wcls = add(F.wcls.data(), F.wcls.size());
+    const size_t i_r32 = add(F.r32.data(), sizeof(float4) * F.r32.size());
+    const size_t i_r64 = add(F.r64.data(), sizeof(double4_32a) * F.r64.size());
+    const size_t i_group = add(F.group.data(), sizeof(uint4) * F.group.size());
     const size_t i_Tj = add(H.Tj.data(), sizeof(double) * MM * ns_pad);
     const size_t i_Tjk = add(H.Tjk.data(), sizeof(double) * MM * ns_pad);
     const size_t i_Tjf = add(Tjf.data(), sizeof(float) * MM * ns_pad);
@@ -471,15 +513,10 @@ extern "C" vmc_status vmc_build_screened_lists(vmc_ctx *ctx, int M, const double
     }
     auto P = [&](size_t idx) { return (void *)(base + pcs[idx].off); };
     v.unit_tab = (const uint4 *)P(i_tab);
-    v.s_off = (const uint32_t *)P(i_s_off); v.s_len = (const uint32_t *)P(i_s_len);
     v.s_owner = (const uint32_t *)P(i_s_owner); v.s_a = (const uint16_t *)P(i_s_a);
-    v.s_rec32 = (const float4 *)P(i_s_r32); v.s_rec64 = (const double4_32a *)P(i_s_r64);
-    v.ds_off = (const uint32_t *)P(i_ds_off); v.ds_len = (const uint32_t *)P(i_ds_len);
-    v.ds_ab = (const uint32_t *)P(i_ds_ab); v.ds_owner = (const uint32_t *)P(i_ds_owner);
-    v.ds_rec32 = (const float4 *)P(i_ds_r32); v.ds_rec64 = (const double4_32a *)P(i_ds_r64);
-    v.do_off = (const uint32_t *)P(i_do_off); v.do_len = (const uint32_t *)P(i_do_len);
-    v.do_ab = (const uint32_t *)P(i_do_ab); v.do_owner = (const uint32_t *)P(i_do_owner);
-    v.do_rec32 = (const float4 *)P(i_do_r32); v.do_rec64 = (const double4_32a *)P(i_do_r64);
+    v.key = (const uint32_t *)P(i_key); v.alive = (const uint32_t *)P(i_alive);
+    v.wcls = (const uint8_t *)P(i_wcls); v.group = (const uint4 *)P(i_group);
+    v.rec32 = (const float4 *)P(i_r32); v.rec64 = (const double4_32a *)P(i_r64);
     v.Tj = (const double *)P(i_Tj); v.Tjk = (const double *)P(i_Tjk);
     v.Tjf = (const float *)P(i_Tjf); v.Tjkf = (const float *)P(i_Tjkf);
     v.Jd = (const double *)P(i_Jd); v.Kd = (const double *)P(i_Kd);
@@ -498,7 +535,7 @@ extern "C" vmc_status vmc_lists_destroy(vmc_lists *L) {
     if (!L) return VMC_OK;
     if (L->dev) cudaFree(L->dev);
     free(L->h_s_key); free(L->h_ds_key); free(L->h_do_key);
-    free(L->h_s_off); free(L->h_ds_off); free(L->h_do_off);
+    free(L->h_s_off); free(L->h_ds_off); free(L->h_do_off); free(L->h_base);
     delete L;
     return VMC_OK;
 }
@@ -550,53 +587,28 @@ __global__ void k_refresh_jastrow(ListsView L, const double *__restrict__ J, dou
         js64[t] = v;
         js32[t] = (float)v;
     }
-    const int64_t tot = 2 * L.ns + 2 * L.nds + L.ndo;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < tot;
-         t += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t tot = (int64_t)L.words * 32;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t key = L.key[e];
+        const int cls = L.wcls[e >> 5], sa = (cls & 1) * M, sb = (cls >> 1) * M;
+        const int A = sa + (int)(key & 0xFFu), I = sa + (int)(key >> 16 & 0xFFu);
+        const int B = sb + (int)(key >> 8 & 0xFFu), Jj = sb + (int)(key >> 24);
+        if (A == I) continue;                    // an unused place
         double lw;
-        if (t < 2 * L.ns) {
-            const int sg = (int)(t / L.ns);
-            const int64_t e = t % L.ns;
-            const int I = sg * M + (int)L.s_owner[e], A = sg * M + L.s_a[e];
+        if (A == B)                              // a single
             lw = -jget(J, N2, A, I) + jget(J, N2, A, A) - jget(J, N2, I, I);
-            const double w = exp(lw);
-            ((double *)&L.s_rec64[e])[1 + sg] = w;
-            ((float *)&L.s_rec32[e])[1 + sg] = (float)w;
-            continue;
-        }
-        int I, Jj, A, B;
-        int64_t e;
-        int cls;
-        if (t < 2 * L.ns + 2 * L.nds) {
-            const int64_t u = t - 2 * L.ns;
-            cls = (int)(u / L.nds);
-            e = u % L.nds;
-            const uint32_t ow = L.ds_owner[e], ab = L.ds_ab[e];
-            I = cls * M + (int)(ow & 0xFFFF); Jj = cls * M + (int)(ow >> 16);
-            A = cls * M + (int)(ab & 0xFFFF); B = cls * M + (int)(ab >> 16);
-        } else {
-            cls = 2;
-            e = t - 2 * L.ns - 2 * L.nds;
-            const uint32_t ow = L.do_owner[e], ab = L.do_ab[e];
-            I = (int)(ow & 0xFFFF); Jj = M + (int)(ow >> 16);
-            A = (int)(ab & 0xFFFF); B = M + (int)(ab >> 16);
-        }
-        lw = -jget(J, N2, A, I) - jget(J, N2, A, Jj) - jget(J, N2, B, I) - jget(J, N2, B, Jj)
-             + jget(J, N2, A, B) + jget(J, N2, I, Jj)
-             + jget(J, N2, A, A) + jget(J, N2, B, B) - jget(J, N2, I, I) - jget(J, N2, Jj, Jj);
+        else
+            lw = -jget(J, N2, A, I) - jget(J, N2, A, Jj) - jget(J, N2, B, I) - jget(J, N2, B, Jj)
+                 + jget(J, N2, A, B) + jget(J, N2, I, Jj)
+                 + jget(J, N2, A, A) + jget(J, N2, B, B) - jget(J, N2, I, I) - jget(J, N2, Jj, Jj);
         const double w = exp(lw);
-        if (cls < 2) {
-            ((double *)&L.ds_rec64[e])[2 + cls] = w;
-            ((float *)&L.ds_rec32[e])[2 + cls] = (float)w;
-        } else {
-            ((double *)&L.do_rec64[e])[2] = w;
-            ((float *)&L.do_rec32[e])[2] = (float)w;
-        }
+        ((double *)&L.rec64[e])[2] = w;
+        ((float *)&L.rec32[e])[2] = (float)w;
     }
 }
 
 vmc_status launch_refresh_jastrow(vmc_ctx *ctx, vmc_lists *L, const double *J) {
-    const int64_t tot = std::max<int64_t>(2 * L->ns + 2 * L->nds + L->ndo, 4 * (int64_t)L->M * L->M);
+    const int64_t tot = std::max<int64_t>((int64_t)L->view.words * 32, 4 * (int64_t)L->M * L->M);
     int blocks = (int)std::min<int64_t>((tot + 255) / 256, 152 * 16);
     double *js64 = (double *)L->jsym;
     float *js32 = (float *)(js64 + 4 * (size_t)L->M * L->M);
