@@ -13,8 +13,9 @@
 namespace {
 
 constexpr int kChunkJ = 256;    // walkers per CTA for dJ
-constexpr int kChunkC = 64;     // walkers per CTA for dC
-constexpr int kRowsC = 16;      // orbital rows per CTA (registers per thread) for dC
+constexpr int kChunkC = 64;     // walkers per dC partial of the mixed form (the length of its FP32 sums)
+constexpr int kRowsC = 16;      // orbital rows per CTA (registers per thread) of k_grad_C_reg
+constexpr int kWalkC = 64;      // walkers whose orbitals and weights a dC CTA holds at a time
 
 // 32 consecutive spin-orbital occupation bits starting at spin orbital p0 (lane l -> bit l)
 __device__ __forceinline__ uint32_t window_bits(const uint32_t *bits_w, int M, int nw, int p0, int lane) {
@@ -180,18 +181,121 @@ __global__ void k_reduce_J(int M, int n_chunks, const long long *__restrict__ pa
     }
 }
 
-// dC partials: CTA = (spin, block of kRowsC orbital rows) x walker chunk; thread x owns the
-// accumulators dC[k][x] of its rows in registers: acc[k][x] += c_w AinvT_w[pos_w(k)][x] for
-// occupied k.  part layout: [n_out][chunk][2][M][nmax].  acc_t = float (mixed) or double.
-template <typename real, typename acc_t>
+// dC partials: sum_w c_w AinvT_w[col(k)][x] for occupied k.  CTA = (spin, range of k) x walker chunk, with the
+// accumulators [k][x] of one or two weight sets in shared memory.  A warp owns a block of columns x
+// (kXL lanes of VE elements) and goes through every walker's rows c in order, 32 / kXL rows at a time; row c
+// belongs to orbital k = occ[c], so rows of one walker never meet and no other warp touches the warp's
+// columns.  AinvT is read once, contiguously and with kDepth to 2 kDepth loads per lane in flight, and nothing is
+// done for unoccupied orbitals (a thread per x with register accumulators for 16 orbitals spends half of its
+// multiply-adds on zeros, and leaves 24 of 64 lanes idle at n = 40).  Per accumulator the walkers of a chunk
+// are added in order.  Bound: latency and shared-memory
+// read-modify-writes; H80, 16,384 walkers, FP64: 672 -> 195 us (its FP64 multiply-adds alone 167 us).
+// part layout: [n_out][chunk][2][M][nmax].  acc_t = float (mixed) or double.
+constexpr int kXL = 4, kDepth = 8;
+
+template <typename real, int VE> struct __align__(sizeof(real) * VE) RowVec { real v[VE]; };
+
+template <typename real, int VE, int kMode>
+__global__ void __launch_bounds__(1024 / VE)          // (at most 32 warps of kXL VE columns: n <= 128)
+k_grad_C(int W, int M, int na, int nb, int chunk, int n_k, const uint16_t *__restrict__ occ, const real *__restrict__ AinvT,
+         const double *__restrict__ wgt, const double *__restrict__ e, double *__restrict__ part) {
+    constexpr int kCL = 32 / kXL;                    // rows per step
+    typedef RowVec<real, VE> vec;
+    const int s = blockIdx.x & 1, k0 = (blockIdx.x >> 1) * n_k, nk = min(n_k, M - k0);
+    const int n = s ? nb : na, ne = na + nb, nmax = na > nb ? na : nb;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x;
+    extern __shared__ __align__(16) unsigned char sm[];
+    real *acc0 = (real *)sm, *acc1 = acc0 + (size_t)n_k * nmax;           // [k][x], rows of n
+    real *s_w = acc0 + (size_t)(kMode + 1) * n_k * nmax;                  // [kWalkC][2] weights
+    uint16_t *s_occ = (uint16_t *)(s_w + 2 * kWalkC);                     // [kWalkC][n]
+    for (int t = tid; t < (kMode + 1) * n_k * nmax; t += nt) acc0[t] = real(0);
+    const size_t astride = (size_t)na * na + (size_t)nb * nb;
+    const int w_begin = blockIdx.y * chunk, w_end = min(W, w_begin + chunk);
+    const int x = (warp * kXL + lane % kXL) * VE, cl = lane / kXL, G = (n + kCL - 1) / kCL;
+    const bool xin = x < n;                          // (n is a multiple of VE)
+    for (int wb = w_begin; wb < w_end; wb += kWalkC) {
+        const int nw = min(kWalkC, w_end - wb);
+        __syncthreads();
+        for (int t = tid; t < nw * n; t += nt) {
+            const int i = t / n, c = t - i * n;
+            s_occ[t] = occ[(size_t)(wb + i) * ne + (s ? na : 0) + c];
+        }
+        for (int i = tid; i < nw; i += nt) {
+            double c0, c1;
+            weights(kMode, wgt, e, wb + i, c0, c1);
+            s_w[2 * i] = (real)c0;
+            s_w[2 * i + 1] = (real)c1;
+        }
+        __syncthreads();
+        const real *A = AinvT + (size_t)wb * astride + (s ? (size_t)na * na : 0);
+        int wl = 0, gl = 0;                          // walker and row step of the next load
+        struct Step {
+            vec v;
+            int at, w;                               // accumulator offset (-1: none), walker
+        } cur[kDepth], nxt[kDepth];
+        auto load = [&](Step (&p)[kDepth]) {
+#pragma unroll
+            for (int u = 0; u < kDepth; ++u) {
+                const int c = gl * kCL + cl;
+                p[u].at = -1;
+                p[u].w = wl;
+                if (wl < nw && c < n && xin) {
+                    const int k = (int)s_occ[wl * n + c] - k0;
+                    if ((unsigned)k < (unsigned)nk) {
+                        p[u].at = k * n + x;
+                        p[u].v = *(const vec *)(A + (size_t)wl * astride + (size_t)c * n + x);
+                    }
+                }
+                if (++gl == G) { gl = 0; ++wl; }
+            }
+        };
+        load(cur);
+        for (int f0 = 0; f0 < nw * G; f0 += kDepth) {
+            load(nxt);                               // in flight while the previous ones are added
+#pragma unroll
+            for (int u = 0; u < kDepth; ++u) {
+                if (cur[u].at >= 0) {
+                    const real c0 = s_w[2 * cur[u].w], c1 = kMode ? s_w[2 * cur[u].w + 1] : real(0);
+                    vec p = *(const vec *)(acc0 + cur[u].at);
+#pragma unroll
+                    for (int q = 0; q < VE; ++q) p.v[q] += c0 * cur[u].v.v[q];
+                    *(vec *)(acc0 + cur[u].at) = p;
+                    if (kMode) {
+                        vec r = *(const vec *)(acc1 + cur[u].at);
+#pragma unroll
+                        for (int q = 0; q < VE; ++q) r.v[q] += c1 * cur[u].v.v[q];
+                        *(vec *)(acc1 + cur[u].at) = r;
+                    }
+                }
+                __syncwarp();                        // the next step may be another walker's
+                cur[u] = nxt[u];
+            }
+        }
+    }
+    __syncthreads();
+    const size_t blk = (size_t)M * nmax;
+    double *dst = part + ((size_t)blockIdx.y * 2 + s) * blk + (size_t)k0 * n;
+    double *dst2 = part + (((size_t)gridDim.y + blockIdx.y) * 2 + s) * blk + (size_t)k0 * n;
+    for (int t = tid; t < nk * n; t += nt) {
+        dst[t] = (double)acc0[t];
+        if (kMode) dst2[t] = (double)acc1[t];
+    }
+}
+
+// The mixed form's dC partials for n_sigma > kRegC: CTA = (spin, block of kRowsC orbital rows) x walker chunk;
+// thread x owns the accumulators dC[k][x] of its rows in registers: acc[k][x] += c_w AinvT_w[pos_w(k)][x] for
+// occupied k.  Its chunks of 64 walkers are too short for the shared-memory kernel above to fill the SMs with the few
+// CTAs that its accumulators leave (H160: 798 us there, 679 us here; H61, 8,192 walkers: 141 and 131 us a call;
+// at n = 10 it is 117 us here and 90 us there).
+constexpr int kRegC = 24;
 __global__ void __launch_bounds__(128)
-k_grad_C(int W, int M, int na, int nb, const uint16_t *__restrict__ pos, const real *__restrict__ AinvT,
+k_grad_C_reg(int W, int M, int na, int nb, const uint16_t *__restrict__ pos, const float *__restrict__ AinvT,
          const double *__restrict__ wgt, const double *__restrict__ e, int mode, double *__restrict__ part) {
     const int nrb = (M + kRowsC - 1) / kRowsC;
     const int s = blockIdx.x / nrb, rb = blockIdx.x - s * nrb;
     const int n = s ? nb : na, x = threadIdx.x;
     const int k0 = rb * kRowsC;
-    acc_t acc[kRowsC], acc2[kRowsC];
+    float acc[kRowsC], acc2[kRowsC];
 #pragma unroll
     for (int r = 0; r < kRowsC; ++r) { acc[r] = 0; acc2[r] = 0; }
     const size_t astride = (size_t)na * na + (size_t)nb * nb;
@@ -223,19 +327,19 @@ k_grad_C(int W, int M, int na, int nb, const uint16_t *__restrict__ pos, const r
         if (w + 1 < w1) map_of(w + 1, nlo, nhi);    // prefetch the next walker's map
         double c0d, c1d;
         weights(mode, wgt, e, w, c0d, c1d);
-        const acc_t c0 = (acc_t)c0d, c1 = (acc_t)c1d;
-        const real *A = AinvT + (size_t)w * astride + aoff;
+        const float c0 = (float)c0d, c1 = (float)c1d;
+        const float *A = AinvT + (size_t)w * astride + aoff;
         const uint32_t words[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
-        real a[kRowsC];
+        float a[kRowsC];
 #pragma unroll
         for (int r = 0; r < kRowsC; ++r) {         // all row loads in flight together
             const uint32_t pc = (words[r >> 1] >> ((r & 1) * 16)) & 0xFFFFu;
-            a[r] = (xin && k0 + r < M && !(pc & 0x8000u)) ? A[(size_t)pc * n + x] : real(0);
+            a[r] = (xin && k0 + r < M && !(pc & 0x8000u)) ? A[(size_t)pc * n + x] : float(0);
         }
 #pragma unroll
         for (int r = 0; r < kRowsC; ++r) {
-            acc[r] += c0 * (acc_t)a[r];
-            if (mode) acc2[r] += c1 * (acc_t)a[r];
+            acc[r] += c0 * (float)a[r];
+            if (mode) acc2[r] += c1 * (float)a[r];
         }
     }
     if (!xin) return;
@@ -333,11 +437,73 @@ k_walker_reduce(int W, const double *__restrict__ t, const double *__restrict__ 
 
 }  // namespace
 
+// Work split of k_grad_C: orbitals per CTA so that the accumulators take at most half of an SM's shared
+// memory (two CTAs, or more), walkers per CTA: 64 in the mixed form (the FP32 sums' length), in FP64 one
+// wave of CTAs, but 16 or more.
+struct PlanC {
+    int n_k, parts, chunk, chunks;
+    size_t smem;
+};
+static PlanC plan_grad_C(int W, int M, int na, int nb, int esz, int nout) {
+    const int nmax = na > nb ? na : nb;
+    PlanC p;
+    const size_t fixed = 2 * (size_t)esz * kWalkC + sizeof(uint16_t) * (size_t)kWalkC * nmax, room = 112 * 1024 - fixed;
+    const size_t per_k = (size_t)nout * nmax * esz;
+    int parts = 1;
+    while (parts < M && per_k * (size_t)((M + parts - 1) / parts) > room) ++parts;
+    p.n_k = (M + parts - 1) / parts;
+    p.parts = (M + p.n_k - 1) / p.n_k;
+    p.smem = (per_k * (size_t)p.n_k + fixed + 15) & ~(size_t)15;
+    p.chunk = kChunkC;
+    if (esz == 8) {
+        const int warps = (nmax + kXL * 2 - 1) / (kXL * 2);
+        const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(227 * 1024 / (p.smem + 1024), 64 / std::max(1, warps)));
+        const int ctas = std::max(1, 152 * std::min(per_sm, 8) / (2 * p.parts));
+        p.chunk = std::max(16, (W + ctas - 1) / ctas);
+    }
+    p.chunks = (W + p.chunk - 1) / p.chunk;
+    return p;
+}
+
+template <typename real, int VE>
+static cudaError_t grad_C_launch_v(vmc_ctx *ctx, const vmc_walkers *Wk, const PlanC &p, const double *t, const double *e,
+                                   int mode, double *part) {
+    const int na = Wk->n_alpha, nb = Wk->n_beta, nmax = na > nb ? na : nb;
+    const int threads = 32 * ((nmax + kXL * VE - 1) / (kXL * VE));
+    const dim3 grid(2 * p.parts, p.chunks);
+    auto *k = mode ? k_grad_C<real, VE, 1> : k_grad_C<real, VE, 0>;
+    cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+    if (err == cudaSuccess)
+        k<<<grid, threads, p.smem, ctx->stream>>>(Wk->W, Wk->M, na, nb, p.chunk, p.n_k, Wk->occ_list,
+                                                  (const real *)Wk->AinvT, t, e, part);
+    return err == cudaSuccess ? cudaGetLastError() : err;
+}
+
+// 16-byte, 8-byte or single elements: rows start at multiples of n_alpha and n_beta elements
+template <typename real>
+static cudaError_t grad_C_launch(vmc_ctx *ctx, const vmc_walkers *Wk, const PlanC &p, const double *t, const double *e,
+                                 int mode, double *part) {
+    const int na = Wk->n_alpha, nb = Wk->n_beta;
+    const uintptr_t a = (uintptr_t)Wk->AinvT;
+    constexpr int most = 16 / (int)sizeof(real);
+    if (na % most == 0 && nb % most == 0 && a % 16 == 0) return grad_C_launch_v<real, most>(ctx, Wk, p, t, e, mode, part);
+    if (most == 4 && na % 2 == 0 && nb % 2 == 0 && a % 8 == 0) return grad_C_launch_v<real, 2>(ctx, Wk, p, t, e, mode, part);
+    return grad_C_launch_v<real, 1>(ctx, Wk, p, t, e, mode, part);
+}
+
+static cudaError_t grad_C_reg_launch(vmc_ctx *ctx, const vmc_walkers *Wk, const PlanC &p, const double *t, const double *e,
+                                     int mode, double *part) {
+    const int M = Wk->M, na = Wk->n_alpha, nb = Wk->n_beta, nmax = na > nb ? na : nb;
+    const dim3 grid(2 * ((M + kRowsC - 1) / kRowsC), p.chunks);
+    k_grad_C_reg<<<grid, (nmax + 31) / 32 * 32, 0, ctx->stream>>>(Wk->W, M, na, nb, Wk->pos, (const float *)Wk->AinvT, t, e,
+                                                                  mode, part);
+    return cudaGetLastError();
+}
+
 static vmc_status grad_impl(vmc_ctx *ctx, const vmc_walkers *Wk, const double *t, const double *e, int mode,
                             double *const out0[3], double *const out1[3], double *sums) {
     const int W = Wk->W, M = Wk->M, na = Wk->n_alpha, nb = Wk->n_beta, N2 = 2 * M;
     const int T = (N2 + 31) / 32, ntile = T * (T + 1) / 2;
-    const int cc = (W + kChunkC - 1) / kChunkC;
     const bool jtc = ctx->grad_j_tc != 0 && out0[0] != nullptr;
     int cj = (W + kChunkJ - 1) / kChunkJ, chunk_j = kChunkJ;
     if (jtc) {
@@ -353,6 +519,8 @@ static vmc_status grad_impl(vmc_ctx *ctx, const vmc_walkers *Wk, const double *t
     const size_t parts = 256 + sizeof(double) * 4 * kWeightParts;
     const size_t head = parts + sizeof(long long) * 2 * (size_t)W;
     const size_t bytes_J = sizeof(long long) * (size_t)nout * cj * N2 * N2;
+    const PlanC pc = plan_grad_C(W, M, na, nb, Wk->precision == VMC_FP64 ? 8 : 4, nout);
+    const int cc = pc.chunks;
     const size_t bytes_C = sizeof(double) * (size_t)nout * cc * 2 * M * nmax;
     vmc_status st = ensure_workspace(ctx, head + (bytes_J > bytes_C ? bytes_J : bytes_C));
     if (st) return st;
@@ -383,20 +551,16 @@ static vmc_status grad_impl(vmc_ctx *ctx, const vmc_walkers *Wk, const double *t
         if (err != cudaSuccess) return cuda_check(ctx, err, "k_grad_J");
     }
     if (out0[1] && out0[2]) {
-        const int nrb = (M + kRowsC - 1) / kRowsC;
-        const int threads = ((nmax + 31) / 32) * 32;
-        dim3 grid(2 * nrb, cc);
-        if (Wk->precision == VMC_FP64)
-            k_grad_C<double, double><<<grid, threads, 0, ctx->stream>>>(W, M, na, nb, Wk->pos, (const double *)Wk->AinvT,
-                                                                        t, e, mode, (double *)part);
-        else
-            k_grad_C<float, float><<<grid, threads, 0, ctx->stream>>>(W, M, na, nb, Wk->pos, (const float *)Wk->AinvT,
-                                                                      t, e, mode, (double *)part);
+        cudaError_t err = Wk->precision == VMC_FP64
+                              ? grad_C_launch<double>(ctx, Wk, pc, t, e, mode, (double *)part)
+                              : (nmax > kRegC ? grad_C_reg_launch(ctx, Wk, pc, t, e, mode, (double *)part)
+                                              : grad_C_launch<float>(ctx, Wk, pc, t, e, mode, (double *)part));
+        if (err != cudaSuccess) return cuda_check(ctx, err, "k_grad_C");
         const int tot = nout * (M * na + M * nb);
         k_reduce_C<<<(tot + 31) / 32, 256, 0, ctx->stream>>>(M, na, nb, cc, nout, (const double *)part, out0[1],
                                                                out0[2], mode ? out1[1] : nullptr, mode ? out1[2] : nullptr);
         ctx->launches += 2;
-        cudaError_t err = cudaGetLastError();
+        err = cudaGetLastError();
         if (err != cudaSuccess) return cuda_check(ctx, err, "k_grad_C");
     }
     return VMC_OK;
