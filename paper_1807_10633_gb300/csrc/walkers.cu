@@ -69,62 +69,6 @@ __device__ void gj_invert(double *B, double *X, int n, int ld, double *colk, int
     }
 }
 
-// LU with partial pivoting in shared memory; returns log|det| and sign (0 if singular).
-__device__ void lu_logdet(double *B, int n, int ld, int *s_piv, double *s_acc, double *logabs,
-                          int *sign) {
-    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
-    __shared__ double s_log;
-    __shared__ int s_sgn;
-    if (tid == 0) { s_log = 0.0; s_sgn = 1; }
-    __syncthreads();
-    for (int k = 0; k < n; ++k) {
-        if (warp == 0) {
-            double best = -1.0;
-            int idx = k;
-            for (int r = k + lane; r < n; r += 32) {
-                const double v = fabs(B[r * ld + k]);
-                if (v > best) { best = v; idx = r; }
-            }
-#pragma unroll
-            for (int m = 16; m >= 1; m >>= 1) {
-                const double ob = __shfl_xor_sync(0xffffffffu, best, m);
-                const int oi = __shfl_xor_sync(0xffffffffu, idx, m);
-                if (ob > best || (ob == best && oi < idx)) { best = ob; idx = oi; }
-            }
-            if (lane == 0) *s_piv = idx;
-        }
-        __syncthreads();
-        const int p = *s_piv;
-        if (p != k) {
-            for (int c = tid; c < n; c += nt) {
-                const double t = B[k * ld + c];
-                B[k * ld + c] = B[p * ld + c];
-                B[p * ld + c] = t;
-            }
-        }
-        __syncthreads();
-        const double d = B[k * ld + k];
-        if (tid == 0) {
-            if (p != k) s_sgn = -s_sgn;
-            if (d == 0.0) s_sgn = 0;
-            else {
-                s_log += log(fabs(d));
-                if (d < 0) s_sgn = -s_sgn;
-            }
-        }
-        for (int t = tid; t < (n - k - 1) * (n - k); t += nt) {
-            const int r = k + 1 + t / (n - k), c = k + t % (n - k);
-            if (c == k) continue;
-            const double f = B[r * ld + k] / (d == 0.0 ? 1.0 : d);
-            B[r * ld + c] -= f * B[k * ld + c];
-        }
-        __syncthreads();
-    }
-    (void)s_acc;
-    *logabs = s_log;
-    *sign = s_sgn;
-}
-
 template <typename real>
 __global__ void __launch_bounds__(VMC_THREADS)
 k_init_tables(int M, int na, int nb, const double *__restrict__ Ca, const double *__restrict__ Cb,
@@ -204,44 +148,13 @@ __device__ void refresh_orbitals(int w, int sg, int M, int na, int nb, const uin
                                  uint16_t *virt_list, uint16_t *pos_all, uint32_t *occ_bits, uint16_t *s_occ,
                                  uint16_t *s_virt, uint8_t *mark);
 
-// Mixed form: LU of C_occ^T with partial pivoting in FP64 (in shared memory), then the inverse
-// from the factors and G = C C_occ^-1 in FP32, the precision these tables are kept in.
-// Shared memory: one n x (n+1) FP64 buffer; after the factorisation it is reused as two FP32
-// n x (n+1) arrays (factors, inverse), so four CTAs fit on an SM.
-__global__ void __launch_bounds__(VMC_THREADS)
-k_init_tables_mixed(int M, int na, int nb, const double *__restrict__ Ca, const double *__restrict__ Cb,
-                    const float *__restrict__ Cf, uint16_t *occ_list, uint16_t *virt_list, uint16_t *pos_all,
-                    uint32_t *occ_bits, float *G, float *AinvT, unsigned *status, int do_g) {
-    const int w = blockIdx.x, sg = blockIdx.y;
-    const int n = sg ? nb : na, nv = M - n;
-    const int ne = na + nb, nw = (M + 31) / 32;
-    const double *C = sg ? Cb : Ca;
-    const float *Csf = Cf + (sg ? (size_t)M * na : 0);     // FP32 copy of C^sigma
+// LU with partial pivoting of the n x n FP64 matrix B in shared memory (row stride ld) by the whole CTA:
+// P B = L U, rows left in place; returns the row list rl (rl[k] = the row that is pivot k; perm, with
+// perm[k] = k on entry, or perm2).  Look-ahead: while warps 1.. update columns k+2.. of step k, warp 0
+// updates column k+1, picks the pivot of step k+1 into the other row list and scales its
+// multipliers, so the serial pivot work overlaps the FP64 update.  A zero pivot sets *sing.  Ends with a barrier.
+__device__ __forceinline__ const int *lu_factor(double *B, int n, int ld, int *perm, int *perm2, int *sing) {
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
-    extern __shared__ double sm[];
-    const int ld = n + 1;
-    double *B = sm;                               // n x ld FP64: LU factors
-    float *LUf = (float *)sm;                     // n x ld FP32 (aliases B after the factorisation)
-    float *Y = LUf + (size_t)n * ld;              // n x ld FP32
-    __shared__ uint16_t s_occ[VMC_MAX_M], s_virt[VMC_MAX_M];
-    __shared__ uint8_t mark[VMC_MAX_M];
-    __shared__ int perm[VMC_MAX_M];
-    __shared__ int s_sing;
-    (void)ne; (void)nw; (void)nv;
-    if (tid == 0) s_sing = 0;
-    // occupied/virtual lists, occupation words and the orbital map (ends with a barrier after s_occ)
-    refresh_orbitals(w, sg, M, na, nb, occ_list, virt_list, pos_all, occ_bits, s_occ, s_virt, mark);
-    for (int c = tid; c < n; c += nt) perm[c] = c;
-    for (int t = tid; t < n * n; t += nt) {       // B = C_occ^T: B[x][c] = C[occ[c]][x], read along rows of C
-        const int c = t / n, x = t % n;
-        B[x * ld + c] = C[(size_t)s_occ[c] * n + x];
-    }
-    __syncthreads();
-    // ---- LU with partial pivoting, FP64: P B = L U, rows left in place (row list rl: rl[k] = the
-    //      row that is pivot k).  Look-ahead: while warps 1.. update columns k+2.. of step k, warp 0
-    //      updates column k+1, picks the pivot of step k+1 into the other row list and scales its
-    //      multipliers, so the serial pivot work overlaps the FP64 update.
-    __shared__ int perm2[VMC_MAX_M];
     auto pivot = [&](int k, const int *rin, int *rout) {      // warp 0 only
         for (int r = lane; r < n; r += 32) rout[r] = rin[r];
         __syncwarp();
@@ -263,7 +176,7 @@ k_init_tables_mixed(int M, int na, int nb, const double *__restrict__ Ca, const 
         __syncwarp();
         const double d = B[rout[k] * ld + k];
         const bool zero = ((unsigned long long)__double_as_longlong(d) << 1) == 0ull;   // +-0
-        if (zero && lane == 0) s_sing = 1;
+        if (zero && lane == 0) *sing = 1;
         const double dinv = zero ? 1.0 : __drcp_rn(d);
         for (int r = k + 1 + lane; r < n; r += 32) B[rout[r] * ld + k] *= dinv;
     };
@@ -297,7 +210,44 @@ k_init_tables_mixed(int M, int na, int nb, const double *__restrict__ Ca, const 
         __syncthreads();
         int *t = cur; cur = nxt; nxt = t;
     }
-    const int *rl = cur;
+    return cur;
+}
+
+// Mixed form: LU of C_occ^T with partial pivoting in FP64 (in shared memory), then the inverse
+// from the factors and G = C C_occ^-1 in FP32, the precision these tables are kept in.
+// Shared memory: one n x (n+1) FP64 buffer; after the factorisation it is reused as two FP32
+// n x (n+1) arrays (factors, inverse), so four CTAs fit on an SM.
+__global__ void __launch_bounds__(VMC_THREADS)
+k_init_tables_mixed(int M, int na, int nb, const double *__restrict__ Ca, const double *__restrict__ Cb,
+                    const float *__restrict__ Cf, uint16_t *occ_list, uint16_t *virt_list, uint16_t *pos_all,
+                    uint32_t *occ_bits, float *G, float *AinvT, unsigned *status, int do_g) {
+    const int w = blockIdx.x, sg = blockIdx.y;
+    const int n = sg ? nb : na, nv = M - n;
+    const int ne = na + nb, nw = (M + 31) / 32;
+    const double *C = sg ? Cb : Ca;
+    const float *Csf = Cf + (sg ? (size_t)M * na : 0);     // FP32 copy of C^sigma
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
+    extern __shared__ double sm[];
+    const int ld = n + 1;
+    double *B = sm;                               // n x ld FP64: LU factors
+    float *LUf = (float *)sm;                     // n x ld FP32 (aliases B after the factorisation)
+    float *Y = LUf + (size_t)n * ld;              // n x ld FP32
+    __shared__ uint16_t s_occ[VMC_MAX_M], s_virt[VMC_MAX_M];
+    __shared__ uint8_t mark[VMC_MAX_M];
+    __shared__ int perm[VMC_MAX_M];
+    __shared__ int s_sing;
+    (void)ne; (void)nw; (void)nv;
+    if (tid == 0) s_sing = 0;
+    // occupied/virtual lists, occupation words and the orbital map (ends with a barrier after s_occ)
+    refresh_orbitals(w, sg, M, na, nb, occ_list, virt_list, pos_all, occ_bits, s_occ, s_virt, mark);
+    for (int c = tid; c < n; c += nt) perm[c] = c;
+    for (int t = tid; t < n * n; t += nt) {       // B = C_occ^T: B[x][c] = C[occ[c]][x], read along rows of C
+        const int c = t / n, x = t % n;
+        B[x * ld + c] = C[(size_t)s_occ[c] * n + x];
+    }
+    __syncthreads();
+    __shared__ int perm2[VMC_MAX_M];
+    const int *rl = lu_factor(B, n, ld, perm, perm2, &s_sing);
     if (s_sing && tid == 0) atomicOr(status, VMC_DEV_SINGULAR);
     // reciprocals of U's diagonal (one FP64 division per row, not per element; n <= 128)
     __shared__ double rdiag[VMC_MAX_M / 2];
@@ -860,58 +810,118 @@ k_init_sums(ListsView L, int na, int nb, const real *__restrict__ Jsym, const ui
     }
 }
 
+// ln C[n] = sum_{p<q} J_pq n_p n_q + sum_p J_pp n_p over occupied spin orbitals s_so[0 .. ne): this thread's
+// terms t, t + stride, ...
+__device__ __forceinline__ double jastrow_terms(const double *__restrict__ J, int N2, const int *s_so, int ne, int t, int stride) {
+    double part = 0.0;
+    for (; t < ne * ne; t += stride) {
+        const int x = t / ne, y = t - x * ne;
+        if (y >= x) part += jget(J, N2, s_so[x], s_so[y]);
+    }
+    return part;
+}
+
+// ln|psi|, n_sigma > 32: one CTA per walker, each spin's determinant by the LU in shared memory.
 __global__ void __launch_bounds__(VMC_THREADS)
 k_log_psi(int M, int na, int nb, const double *__restrict__ Ca, const double *__restrict__ Cb,
           const double *__restrict__ J, const uint16_t *occ_list, double *out, unsigned *status) {
     const int w = blockIdx.x, ne = na + nb, N2 = 2 * M;
     const int tid = threadIdx.x, nt = blockDim.x;
     extern __shared__ double sm[];
-    __shared__ int s_so[2 * VMC_MAX_M];
-    __shared__ int s_piv;
+    __shared__ int s_so[2 * VMC_MAX_M], perm[VMC_MAX_M], perm2[VMC_MAX_M];
+    __shared__ int s_sing;
     __shared__ double red[VMC_WARPS];
     const uint16_t *occ = occ_list + (size_t)w * ne;
     for (int c = tid; c < ne; c += nt) s_so[c] = (c < na ? 0 : M) + occ[c];
+    if (tid == 0) s_sing = 0;
     __syncthreads();
-    // ln C[n] = sum_{p<q} J_pq n_p n_q + sum_p J_pp n_p over the occupied spin orbitals
-    double part = 0.0;
-    for (int t = tid; t < ne * ne; t += nt) {
-        const int x = t / ne, y = t % ne;
-        if (y < x) continue;
-        part += jget(J, N2, s_so[x], s_so[y]);
+    double part = jastrow_terms(J, N2, s_so, ne, tid, nt);
+    for (int sg = 0; sg < 2; ++sg) {
+        const int n = sg ? nb : na, ld = n + 1;
+        if (n == 0) continue;
+        const double *C = sg ? Cb : Ca;
+        __syncthreads();
+        for (int t = tid; t < n * n; t += nt) {
+            const int r = t / n, x = t - r * n;
+            sm[r * ld + x] = C[(size_t)occ[(sg ? na : 0) + r] * n + x];
+        }
+        for (int k = tid; k < n; k += nt) perm[k] = k;
+        __syncthreads();
+        const int *rl = lu_factor(sm, n, ld, perm, perm2, &s_sing);
+        for (int k = tid; k < n; k += nt) part += log(fabs(sm[rl[k] * ld + k]));
     }
     part = warp_sum_f64(part);
     if ((tid & 31) == 0) red[tid >> 5] = part;
     __syncthreads();
-    double total = 0.0;
-    if (tid == 0)
-        for (int k = 0; k < (nt >> 5); ++k) total += red[k];
-    int sgn_total = 1;
-    for (int sg = 0; sg < 2; ++sg) {
-        const int n = sg ? nb : na;
-        if (n == 0) continue;
-        const double *C = sg ? Cb : Ca;
-        const int ld = n + 1;
-        __syncthreads();
-        for (int t = tid; t < n * n; t += nt) {
-            const int r = t / n, x = t % n;
-            sm[r * ld + x] = C[(size_t)occ[(sg ? na : 0) + r] * n + x];
-        }
-        __syncthreads();
-        double la;
-        int sgn;
-        lu_logdet(sm, n, ld, &s_piv, nullptr, &la, &sgn);
-        if (tid == 0) {
-            total += la;
-            sgn_total *= sgn;
-        }
-    }
     if (tid == 0) {
-        if (sgn_total == 0) {
-            atomicOr(status, VMC_DEV_SINGULAR);
-            out[w] = -INFINITY;
-        } else {
-            out[w] = total;
+        double total = 0.0;
+        for (int k = 0; k < (nt >> 5); ++k) total += red[k];
+        if (s_sing) atomicOr(status, VMC_DEV_SINGULAR);
+        out[w] = s_sing ? -INFINITY : total;
+    }
+}
+
+// ln|psi|, n_sigma <= NP <= 32: a warp per walker and spin, lane = row, the row in registers.  Step k: the
+// unused row with the largest |a_k| (keys compared as integers; NaN lowest, ties to the lowest row) is
+// broadcast element by element and eliminated from the other unused rows.  At these sizes the CTA-wide
+// elimination is barriers and latency: 4,096 walkers of H40 took 952 us with it (one FP64 division and an
+// integer division per updated element), 130 us with this kernel.
+constexpr int kLogWarps = 8;     // four walkers per CTA
+
+template <int NP>
+__global__ void __launch_bounds__(kLogWarps * 32)
+k_log_psi_warp(int W, int M, int na, int nb, const double *__restrict__ Ca, const double *__restrict__ Cb,
+               const double *__restrict__ J, const uint16_t *occ_list, double *out, unsigned *status) {
+    __shared__ int s_so[kLogWarps / 2][64];
+    __shared__ double s_sum[kLogWarps];
+    __shared__ int s_zero[kLogWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, ww = warp >> 1, sg = warp & 1;
+    const int w = blockIdx.x * (kLogWarps / 2) + ww, ne = na + nb, n = sg ? nb : na;
+    const bool in = w < W;
+    const uint16_t *occ = occ_list + (size_t)w * ne;
+    if (in && sg == 0)
+        for (int c = lane; c < ne; c += 32) s_so[ww][c] = (c < na ? 0 : M) + occ[c];
+    __syncthreads();
+    double part = in ? jastrow_terms(J, 2 * M, s_so[ww], ne, sg * 32 + lane, 64) : 0.0;
+    bool zero = false;
+    if (in && n > 0) {
+        const double *row = (sg ? Cb : Ca) + (size_t)(lane < n ? occ[(sg ? na : 0) + lane] : 0) * n;
+        double a[NP], dk = 1.0;
+#pragma unroll
+        for (int c = 0; c < NP; ++c) a[c] = lane < n && c < n ? row[c] : 0.0;
+        bool used = lane >= n;
+#pragma unroll
+        for (int k = 0; k < NP; ++k) {
+            if (k < n) {
+                const unsigned long long b = (unsigned long long)__double_as_longlong(a[k]) & 0x7FFFFFFFFFFFFFFFull;
+                const unsigned long long key = used ? 0ull : (b > 0x7FF0000000000000ull ? 1ull : b + 2ull);
+                const uint32_t kh = (uint32_t)(key >> 32), kl = (uint32_t)key;
+                const uint32_t mh = __reduce_max_sync(0xffffffffu, kh);
+                const uint32_t ml = __reduce_max_sync(0xffffffffu, kh == mh ? kl : 0u);
+                const int p = __ffs(__ballot_sync(0xffffffffu, kh == mh && kl == ml && !used)) - 1;
+                const double d = __shfl_sync(0xffffffffu, a[k], p);
+                const bool z = ((unsigned long long)__double_as_longlong(d) << 1) == 0ull;      // +-0
+                zero = zero || z;
+                if (lane == k) dk = d;
+                if (lane == p) used = true;
+                const double f = used ? 0.0 : a[k] * (z ? 1.0 : __drcp_rn(d));
+#pragma unroll
+                for (int c = k + 1; c < NP; ++c)
+                    if (c < n) {
+                        const double q = __shfl_sync(0xffffffffu, a[c], p);
+                        a[c] = fma(-f, q, a[c]);
+                    }
+            }
         }
+        part += lane < n ? log(fabs(dk)) : 0.0;
+    }
+    part = warp_sum_f64(part);
+    if (lane == 0) { s_sum[warp] = part; s_zero[warp] = zero ? 1 : 0; }
+    __syncthreads();
+    if (in && sg == 0 && lane == 0) {
+        const bool z = s_zero[warp] || s_zero[warp + 1];
+        if (z) atomicOr(status, VMC_DEV_SINGULAR);
+        out[w] = z ? -INFINITY : s_sum[warp] + s_sum[warp + 1];
     }
 }
 
@@ -1003,12 +1013,19 @@ vmc_status launch_init_walkers(vmc_ctx *ctx, vmc_lists *L, const vmc_params *P, 
 
 vmc_status launch_log_psi(vmc_ctx *ctx, const vmc_walkers *Wk, const vmc_params *P, double *out) {
     const int nmax = Wk->n_alpha > Wk->n_beta ? Wk->n_alpha : Wk->n_beta;
-    const size_t smem = sizeof(double) * ((size_t)nmax * (nmax + 1) + 1);
-    cudaError_t e = cudaFuncSetAttribute(k_log_psi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-        k_log_psi<<<Wk->W, VMC_THREADS, smem, ctx->stream>>>(Wk->M, Wk->n_alpha, Wk->n_beta, P->C_alpha,
-                                                             P->C_beta, P->J, Wk->occ_list, out,
-                                                             ctx->d_status);
+    cudaError_t e = cudaSuccess;
+    if (nmax <= 32) {
+        const int blocks = (Wk->W + kLogWarps / 2 - 1) / (kLogWarps / 2);
+        auto *k = nmax <= 16 ? k_log_psi_warp<16> : k_log_psi_warp<32>;
+        k<<<blocks, kLogWarps * 32, 0, ctx->stream>>>(Wk->W, Wk->M, Wk->n_alpha, Wk->n_beta, P->C_alpha, P->C_beta, P->J,
+                                                      Wk->occ_list, out, ctx->d_status);
+    } else {
+        const size_t smem = sizeof(double) * ((size_t)nmax * (nmax + 1) + 1);
+        e = cudaFuncSetAttribute(k_log_psi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e == cudaSuccess)
+            k_log_psi<<<Wk->W, VMC_THREADS, smem, ctx->stream>>>(Wk->M, Wk->n_alpha, Wk->n_beta, P->C_alpha, P->C_beta,
+                                                                 P->J, Wk->occ_list, out, ctx->d_status);
+    }
     ctx->launches += 1;
     if (e == cudaSuccess) e = cudaGetLastError();
     return cuda_check(ctx, e, "k_log_psi");
