@@ -1185,6 +1185,12 @@ k_screened_moves(ListsView L, WalkerArgs A, CpsView C, int w_begin, int n_w, int
     }
 }
 
+// Asks for [p, p + bytes) in L2 (whole 16-byte pieces inside it).
+__device__ __forceinline__ void prefetch_l2(const void *p, size_t bytes) {
+    const uintptr_t a = ((uintptr_t)p + 15) & ~(uintptr_t)15, b = ((uintptr_t)p + bytes) & ~(uintptr_t)15;
+    if (b > a) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"((uint32_t)(b - a)) : "memory");
+}
+
 // Move update: one CTA per walker (Sec. III.B): diagonal energy, Jastrow sums, Fock sums, then the
 // rank-1 (singles, opposite-spin doubles) or rank-2 Woodbury (same-spin doubles) update of G and
 // AinvT, and the occupation lists, bits and orbital map.
@@ -1208,6 +1214,13 @@ __device__ __forceinline__ void apply_walker(const ListsView &L, const WalkerArg
     uint16_t *virt = A.virt_list + (size_t)w * (2 * M - ne);
     uint32_t *bits = A.occ_bits_w + (size_t)w * 2 * geo.nw;
     uint16_t *posw = A.pos + (size_t)w * N2;
+    if (tid == 0 && (geo.g_stride + geo.a_stride) * sizeof(real) <= 48 * 1024) {
+        // the rank updates come last and stream G and C_occ^-1: bring them to L2 while the sums are updated, as long
+        // as the walkers of all resident CTAs (six per SM) take less than half of it (choice and update of 4,096
+        // walkers of H100, mixed: 205 -> 181 us; at H160, 102 KB a walker, 1.52 -> 1.63 ms for 32,768)
+        prefetch_l2(Gw, geo.g_stride * sizeof(real));
+        prefetch_l2(Aw, geo.a_stride * sizeof(real));
+    }
     for (int p = tid; p < N2; p += nt) pos[p] = posw[p];
     __syncthreads();
     const int kind = (int)(code & 3), I = (int)((code >> 2) & 1023), Jo = (int)((code >> 12) & 1023);
@@ -1438,8 +1451,10 @@ k_ctmc_apply(ListsView L, WalkerArgs A, CpsView C, const double *__restrict__ J,
     apply_walker<real, kC>(L, A, J, blockIdx.x, move_code, smraw, C);
 }
 
+// (The same bounds: left to itself the compiler took 114 registers, two CTAs per SM; the uneven batch of seven systems
+// of 2,048 walkers: 725 -> 286 us.)
 template <typename real>
-__global__ void __launch_bounds__(512)
+__global__ void __launch_bounds__(256, 6)
 k_ctmc_apply_batched(const SysDesc *__restrict__ sys, int n_sys) {
     extern __shared__ __align__(16) unsigned char smraw[];
     const int t = blockIdx.x;
