@@ -18,7 +18,8 @@ namespace {
 constexpr int kM = 128;          // MMA rows (virtual slots, padded)
 constexpr int kThreads = 256;    // eight warps: warp w reads tensor-memory lanes 32 (w % 4)
 constexpr unsigned kMaxSpin = 1u << 20;
-constexpr int kPreChunks = 8;    // k_g_umma: 16-byte chunks per thread held for the next item
+constexpr int kGThreads = 512;   // k_g_umma: sixteen warps, four per tensor-memory sub-partition
+constexpr int kPreChunks = 4;    // k_g_umma: 16-byte chunks per thread held for the next item
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
     return (uint32_t)__cvta_generic_to_shared(p);
@@ -162,11 +163,14 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t parity) {
 // A and the tensor-memory accumulator are double buffered: staging item i+1 and draining item i-1
 // overlap the MMAs of item i.  Rows n..127 of the A tile are never written: they read whatever
 // follows in shared memory and only feed output rows that are discarded.
-// kPre > 0 (an item's A tile in at most kPre 16-byte chunks per thread, and M <= kThreads): the
+// Bound by staging and the tensor-memory read-back, not by the MMAs (about 1.4 us of an item): sixteen warps, each
+// with a quarter of the accumulator's columns and at most four staged chunks per thread, take 2.37 ms for the
+// 65,536 items of 32,768 H160 walkers, eight warps 3.10 ms.
+// kPre > 0 (an item's A tile in at most kPre 16-byte chunks per thread, and M <= kGThreads): the
 // global loads of item i+1's A tile and orbital map are issued into registers right after item i
 // is staged, so their latency overlaps item i's MMAs and item i-1's epilogue.
 template <int kPre>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kGThreads, 1)
 k_g_umma(int W, int M, int na, int nb, const float *__restrict__ Cf, const uint16_t *__restrict__ pos_all,
          const float *__restrict__ AinvT, float *__restrict__ G, unsigned *status, int lbo_k_major) {
     const int nmax = na > nb ? na : nb;
@@ -216,10 +220,9 @@ k_g_umma(int W, int M, int na, int nb, const float *__restrict__ Cf, const uint1
         const int s = q >= W, w = q - s * W, n = s ? nb : na;
         float *Gw = G + (size_t)w * gstride + (s ? (size_t)(M - na) * na : 0);
         const uint16_t *pq = posb + bq * M;
-        const int wq = warp & 3, half = warp >> 2;
+        const int wq = warp & 3, quarter = warp >> 2;
         const int c = wq * 32 + lane;
-        const int nchunk = Mp / 16, ch0 = half ? (nchunk + 1) / 2 : 0, ch1 = half ? nchunk : (nchunk + 1) / 2;
-        for (int k0 = ch0 * 16; k0 < ch1 * 16; k0 += 16) {
+        for (int k0 = quarter * 16; k0 < Mp; k0 += 16 * (kGThreads / 128)) {
             uint32_t r[16];
             const uint32_t taddr = tmem + (uint32_t)(bq * 256) + ((uint32_t)(wq * 32) << 16) + (uint32_t)k0;
             asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 "
@@ -260,7 +263,7 @@ k_g_umma(int W, int M, int na, int nb, const float *__restrict__ Cf, const uint1
             const float *Cs = Cf + (s ? (size_t)M * na : 0);
             stage_tile<2>(Cs, n, M, n, Kp, Bh, Bl);   // also zeroes rows M..ceil8(M)-1
             const int M8 = (M + 7) & ~7;
-            for (int e = tid; e < (Mp - M8) * Kp; e += kThreads) {   // zero rows ceil8(M)..Mp-1
+            for (int e = tid; e < (Mp - M8) * Kp; e += kGThreads) {   // zero rows ceil8(M)..Mp-1
                 const int r = M8 + e / Kp, k = e % Kp;
                 *(float *)(Bh + core_off(r, k, kp4)) = 0.f;
                 *(float *)(Bl + core_off(r, k, kp4)) = 0.f;
@@ -277,7 +280,7 @@ k_g_umma(int W, int M, int na, int nb, const float *__restrict__ Cf, const uint1
             const float *At = AinvT + (size_t)w * astride + (s ? (size_t)na * na : 0);
             stage_tile<8>(At, n, n, n, Kp, Ah, Al);
             const uint16_t *pw = pos_all + (size_t)w * 2 * M + (size_t)s * M;
-            for (int k = tid; k < M; k += kThreads) posb[buf * M + k] = pw[k];
+            for (int k = tid; k < M; k += kGThreads) posb[buf * M + k] = pw[k];
         }
         asm volatile("fence.proxy.async.shared::cta;");
         asm volatile("tcgen05.fence::before_thread_sync;");
@@ -908,20 +911,20 @@ vmc_status launch_g_umma(vmc_ctx *ctx, const vmc_walkers *Wk, const float *Cf) {
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     // register prefetch of the next item when an A tile fits in kPreChunks 16-byte chunks per thread
     const int nmax = na > nb ? na : nb, Kp = (nmax + 7) & ~7;
-    const bool pre = ((nmax + 7) / 8) * (Kp / 4) * 8 <= kPreChunks * kThreads && M <= kThreads;
+    const bool pre = ((nmax + 7) / 8) * (Kp / 4) * 8 <= kPreChunks * kGThreads && M <= kGThreads;
     const int grid = std::min(nsm, 2 * Wk->W);
     if (pre) {
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_g_umma<kPreChunks>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e == cudaSuccess)
-            k_g_umma<kPreChunks><<<grid, kThreads, smem, ctx->stream>>>(Wk->W, M, na, nb, Cf, Wk->pos,
+            k_g_umma<kPreChunks><<<grid, kGThreads, smem, ctx->stream>>>(Wk->W, M, na, nb, Cf, Wk->pos,
                                                                         (const float *)Wk->AinvT, (float *)Wk->G,
                                                                         ctx->d_status, 1);
     } else {
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_g_umma<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e == cudaSuccess)
-            k_g_umma<0><<<grid, kThreads, smem, ctx->stream>>>(Wk->W, M, na, nb, Cf, Wk->pos, (const float *)Wk->AinvT,
+            k_g_umma<0><<<grid, kGThreads, smem, ctx->stream>>>(Wk->W, M, na, nb, Cf, Wk->pos, (const float *)Wk->AinvT,
                                                                (float *)Wk->G, ctx->d_status, 1);
     }
     ctx->launches += 1;
