@@ -394,7 +394,7 @@ vmc_status vmc_grad_logpsi_noalloc(const vmc_walkers *walkers, const double *d_w
 
 /* Context options.  VMC_OPT_G_TENSOR_CORES (default 1): the refresh forms G = C C_occ^-1 on the
    tcgen05 tensor cores.  Mixed form: TF32 MMAs with a split-precision correction (0: FP32 CUDA
-   cores).  FP64 form (register Gauss-Jordan refresh, n_sigma <= 128): every row of C and of
+   cores).  FP64 form (register Gauss-Jordan refresh, 24 < n_sigma <= 128; below, FP64 FMAs): every row of C and of
    C_occ^-T is scaled by a power of two and split into six BF16 digits of 8 bits, the digit
    products are summed exactly in FP32 and combined in 64-bit integers; G differs from the exact
    product by less than about 2^-43 n_sigma of the product of the two rows' power-of-two scales

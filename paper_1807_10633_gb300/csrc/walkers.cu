@@ -3,6 +3,8 @@
 // and the diagonal energy.  Also ln|psi| per walker (forward of the ln psi autograd function).
 #include <math.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace {
@@ -412,44 +414,62 @@ k_init_tables_mixed(int M, int na, int nb, const double *__restrict__ Ca, const 
 // Mixed form: the Fock sums F[s][e] = h_ai + sum_k n_k^s Tjk[k][e] + n_k^(1-s) Tj[k][e] in FP32 for
 // kFockWalkers walkers per CTA (each table row is read once per CTA), one singles entry per thread;
 // rewritten at every refresh so that the per-move FP32 updates never accumulate beyond one period.
+// Bound by FP32 multiply-adds (4 M per walker and entry); a pair of them (two walkers) per instruction, each
+// rounded as a single one: H160, 32,768 walkers, 3.36 -> 2.77 ms.
 constexpr int kFockWalkers = 16, kFockThreads = 128;
+
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {     // a b + c, element by element
+    unsigned long long x, y, z, d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a.x), "f"(a.y));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(y) : "f"(b.x), "f"(b.y));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(z) : "f"(c.x), "f"(c.y));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(x), "l"(y), "l"(z));
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(d));
+    return r;
+}
 
 __global__ void __launch_bounds__(kFockThreads)
 k_fock_sums_f32(ListsView L, int W, const uint32_t *__restrict__ occ_bits, float *F) {
     const int M = L.M, nw = (M + 31) / 32, w0 = blockIdx.y * kFockWalkers;
-    __shared__ float2 occf[VMC_MAX_M][kFockWalkers];   // (n_alpha, n_beta) of orbital k per walker
+    __shared__ __align__(16) float occf[VMC_MAX_M][2][kFockWalkers];   // n of orbital k per spin and walker
     for (int t = threadIdx.x; t < M * kFockWalkers; t += blockDim.x) {
         const int k = t / kFockWalkers, q = t % kFockWalkers, w = w0 + q;
-        float2 o = make_float2(0.f, 0.f);
+        float a = 0.f, c = 0.f;
         if (w < W) {
             const uint32_t *b = occ_bits + (size_t)w * 2 * nw;
-            o.x = (float)((b[k >> 5] >> (k & 31)) & 1u);
-            o.y = (float)((b[nw + (k >> 5)] >> (k & 31)) & 1u);
+            a = (float)((b[k >> 5] >> (k & 31)) & 1u);
+            c = (float)((b[nw + (k >> 5)] >> (k & 31)) & 1u);
         }
-        occf[k][q] = o;
+        occf[k][0][q] = a;
+        occf[k][1][q] = c;
     }
     __syncthreads();
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= L.ns_pad) return;
     const int64_t np = L.ns_pad;
-    float acc[kFockWalkers][2];
+    float2 fa[kFockWalkers / 2], fb[kFockWalkers / 2];     // two walkers each, per spin
     const float h = e < L.ns ? (float)L.h1[(size_t)L.s_a[e] * M + L.s_owner[e]] : 0.f;
 #pragma unroll
-    for (int q = 0; q < kFockWalkers; ++q) acc[q][0] = acc[q][1] = h;
+    for (int q = 0; q < kFockWalkers / 2; ++q) fa[q] = fb[q] = make_float2(h, h);
     for (int k = 0; k < M; ++k) {
         const float tk = __ldg(L.Tjkf + (size_t)k * np + e), tx = __ldg(L.Tjf + (size_t)k * np + e);
+        const float2 tk2 = make_float2(tk, tk), tx2 = make_float2(tx, tx);
 #pragma unroll
-        for (int q = 0; q < kFockWalkers; ++q) {
-            const float2 o = occf[k][q];
-            acc[q][0] = fmaf(o.x, tk, fmaf(o.y, tx, acc[q][0]));
-            acc[q][1] = fmaf(o.y, tk, fmaf(o.x, tx, acc[q][1]));
+        for (int q = 0; q < kFockWalkers / 4; ++q) {
+            const float4 a = ((const float4 *)occf[k][0])[q], b = ((const float4 *)occf[k][1])[q];
+            const float2 a0 = make_float2(a.x, a.y), a1 = make_float2(a.z, a.w), b0 = make_float2(b.x, b.y), b1 = make_float2(b.z, b.w);
+            fa[2 * q] = fma2(a0, tk2, fma2(b0, tx2, fa[2 * q]));
+            fb[2 * q] = fma2(b0, tk2, fma2(a0, tx2, fb[2 * q]));
+            fa[2 * q + 1] = fma2(a1, tk2, fma2(b1, tx2, fa[2 * q + 1]));
+            fb[2 * q + 1] = fma2(b1, tk2, fma2(a1, tx2, fb[2 * q + 1]));
         }
     }
 #pragma unroll
     for (int q = 0; q < kFockWalkers; ++q)
         if (w0 + q < W) {
-            F[((size_t)(w0 + q) * 2) * np + e] = acc[q][0];
-            F[((size_t)(w0 + q) * 2 + 1) * np + e] = acc[q][1];
+            F[((size_t)(w0 + q) * 2) * np + e] = q & 1 ? fa[q / 2].y : fa[q / 2].x;
+            F[((size_t)(w0 + q) * 2 + 1) * np + e] = q & 1 ? fb[q / 2].y : fb[q / 2].x;
         }
 }
 
@@ -510,11 +530,14 @@ __device__ __forceinline__ unsigned long long abs_inf_bits(float) { return 0x7F8
 __device__ __forceinline__ double rcp_rn(double d) { return __drcp_rn(d); }
 __device__ __forceinline__ float rcp_rn(float d) { return __frcp_rn(d); }
 
-template <typename real, int R>
-__global__ void __launch_bounds__(kGJ * kGJ, sizeof(real) == 4 ? (R <= 5 ? 4 : 2) : (R <= 5 ? 3 : 1))
+// kG: G from the CUDA cores at the end (otherwise on the tensor cores by another kernel; a build without that part
+// needs fewer registers: no spills at three CTAs per SM for n <= 80 in FP64, and six CTAs for n <= 32, whose steps are
+// latency: H61, 5,003 walkers, FP64: 1.10 -> 0.97 ms).
+template <typename real, int R, bool kG>
+__global__ void __launch_bounds__(kGJ * kGJ, sizeof(real) == 4 ? (R <= 5 ? 4 : 2) : (R <= 2 ? 6 : R <= 4 ? 4 : R <= 5 ? 3 : 1))
 k_refresh_gj(int M, int na, int nb, const real *__restrict__ Ca, const real *__restrict__ Cb,
              const uint16_t *occ_list, uint16_t *virt_list, uint16_t *pos_all, uint32_t *occ_bits, real *G,
-             real *AinvT, unsigned *status, int do_g) {
+             real *AinvT, unsigned *status) {
     constexpr int NR = kGJ * R;
     const int w = blockIdx.x, sg = blockIdx.y;
     const int n = sg ? nb : na, nv = M - n, ld = n + 1;
@@ -644,7 +667,7 @@ k_refresh_gj(int M, int na, int nb, const real *__restrict__ Ca, const real *__r
                         (sg ? (size_t)(M - na) * na : 0);
     const size_t aofs = (size_t)w * ((size_t)na * na + (size_t)nb * nb) + (sg ? (size_t)na * na : 0);
     for (int t = tid; t < n * n; t += nt) AinvT[aofs + t] = Y[(t / n) * ld + t % n];
-    if (!do_g) return;   // (mixed form) G is formed on the tensor cores by k_g_umma
+    if (!kG) return;
     // G[s][c] = sum_x C[virt[s]][x] AinvT[c][x]: 4 x 4 register tiles (slots x columns)
     const int ts = (nv + 3) / 4, tc = (n + 3) / 4;
     for (int tile = tid; tile < ts * tc; tile += nt) {
@@ -676,11 +699,11 @@ template <typename real, int R>
 cudaError_t launch_gj_r(vmc_ctx *ctx, const vmc_walkers *Wk, const real *Ca, const real *Cb, int do_g) {
     const int na = Wk->n_alpha, nb = Wk->n_beta, nmax = na > nb ? na : nb;
     const size_t smem = sizeof(real) * (size_t)nmax * (nmax + 1) + 16;
-    cudaError_t e = cudaFuncSetAttribute(k_refresh_gj<real, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    auto *k = do_g ? k_refresh_gj<real, R, true> : k_refresh_gj<real, R, false>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_refresh_gj<real, R><<<dim3(Wk->W, 2), kGJ * kGJ, smem, ctx->stream>>>(
-        Wk->M, na, nb, Ca, Cb, Wk->occ_list, Wk->virt_list, Wk->pos, Wk->occ_bits, (real *)Wk->G,
-        (real *)Wk->AinvT, ctx->d_status, do_g);
+    k<<<dim3(Wk->W, 2), kGJ * kGJ, smem, ctx->stream>>>(Wk->M, na, nb, Ca, Cb, Wk->occ_list, Wk->virt_list, Wk->pos,
+                                                        Wk->occ_bits, (real *)Wk->G, (real *)Wk->AinvT, ctx->d_status);
     return cudaGetLastError();
 }
 
@@ -710,9 +733,16 @@ __global__ void k_convert_c(int M, int na, int nb, const double *__restrict__ Ca
 // (Full init only:) Fock sums F and the diagonal energy, one walker per block.
 constexpr int kSumWalkers = 8;
 
+// A thread takes two neighbouring p (their elements of a row are one load); the warps that M pairs leave over take
+// other walkers of the block: H160, 32,768 walkers, mixed, 0.98 -> 0.65 ms.
+template <typename real> struct Pair;
+template <> struct Pair<float> { typedef float2 type; };
+template <> struct Pair<double> { typedef double2 type; };
+
 template <typename real>
 __global__ void __launch_bounds__(VMC_THREADS)
 k_jastrow_sums(int W, int M, const real *__restrict__ Jsym, const uint32_t *__restrict__ occ_bits, real *S) {
+    typedef typename Pair<real>::type real2;
     const int N2 = 2 * M, nw = (M + 31) / 32, w0 = blockIdx.x * kSumWalkers;
     __shared__ uint32_t bits[kSumWalkers][2 * (VMC_MAX_M / 32)];
     for (int t = threadIdx.x; t < kSumWalkers * 2 * nw; t += blockDim.x) {
@@ -720,14 +750,17 @@ k_jastrow_sums(int W, int M, const real *__restrict__ Jsym, const uint32_t *__re
         bits[k][q] = (w0 + k < W) ? occ_bits[(size_t)(w0 + k) * 2 * nw + q] : 0u;
     }
     __syncthreads();
-    for (int p = threadIdx.x; p < N2; p += blockDim.x) {
-        const real jd = Jsym[(size_t)p * N2 + p];
-        const int sp = p >= M, kp = p - sp * M;
-        for (int k = 0; k < kSumWalkers; ++k) {
+    const real2 *J2 = (const real2 *)Jsym;               // rows of M pairs
+    const int per = (M + 31) / 32 * 32, groups = max(1, (int)blockDim.x / per);    // threads of a walker, walkers at a time
+    const int grp = threadIdx.x / per;
+    for (int h = threadIdx.x - grp * per; h < M && grp < groups; h += per) {
+        const int p = 2 * h;
+        const real jd0 = Jsym[(size_t)p * N2 + p], jd1 = Jsym[(size_t)(p + 1) * N2 + p + 1];
+        for (int k = grp; k < kSumWalkers; k += groups) {
             if (w0 + k >= W) break;
             // only the walker's occupied spin orbitals r, in ascending order (the set bits of its
             // alpha words, then of its beta words): one add each, four row loads in flight at a time
-            real acc = 0;
+            real acc0 = 0, acc1 = 0;
             for (int q = 0; q < 2 * nw; ++q) {
                 uint32_t word = bits[k][q];
                 const int base = q < nw ? 32 * q : M + 32 * (q - nw);
@@ -740,16 +773,20 @@ k_jastrow_sums(int W, int M, const real *__restrict__ Jsym, const uint32_t *__re
                             word &= word - 1u;
                             m = u + 1;
                         }
-                    real j[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) j[u] = u < m ? Jsym[(size_t)r[u] * N2 + p] : real(0);
+                    real2 j[4];
 #pragma unroll
                     for (int u = 0; u < 4; ++u)
-                        if (u < m) acc += j[u];
+                        if (u < m) j[u] = J2[(size_t)r[u] * M + h];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (u < m) { acc0 += j[u].x; acc1 += j[u].y; }
                 }
             }
-            const bool occp = (bits[k][sp * nw + (kp >> 5)] >> (kp & 31)) & 1u;
-            S[(size_t)(w0 + k) * N2 + p] = occp ? acc - jd : acc;
+            auto occ = [&](int x) { const int s = x >= M, y = x - s * M; return (bits[k][s * nw + (y >> 5)] >> (y & 31)) & 1u; };
+            real2 out;
+            out.x = occ(p) ? acc0 - jd0 : acc0;
+            out.y = occ(p + 1) ? acc1 - jd1 : acc1;
+            ((real2 *)S)[(size_t)(w0 + k) * M + h] = out;
         }
     }
 }
@@ -927,6 +964,12 @@ k_log_psi_warp(int W, int M, int na, int nb, const double *__restrict__ Ca, cons
 
 }  // namespace
 
+// FP64 form: up to this n_sigma G is formed with FP64 multiply-adds at the end of the Gauss-Jordan kernel; above it by
+// the digit products, whose persistent kernel takes about 6 us per determinant and SM whatever its size (recompute of
+// 4,096 walkers of H20, n = 10: 376 us against 535; H40, n = 20: 761 and 911; H48, n = 24: 1040 and 1048; H61, n = 31,
+// 5,003 walkers: 1595 and 1477; H80, n = 40: 4290 and 3761).
+constexpr int kCudaCoreG = 24;
+
 vmc_status launch_init_walkers(vmc_ctx *ctx, vmc_lists *L, const vmc_params *P, vmc_walkers *Wk,
                                int full) {
     const int M = Wk->M, na = Wk->n_alpha, nb = Wk->n_beta;
@@ -942,7 +985,7 @@ vmc_status launch_init_walkers(vmc_ctx *ctx, vmc_lists *L, const vmc_params *P, 
     if (reg) {
         if (nmax > kGJ * 8) return set_err(ctx, VMC_ERR_ARG, "n_sigma too large for the register inverse (max 128)");
         if (Wk->precision == VMC_FP64) {
-            const bool oz = ctx->g_tensor_cores && g_ozaki_ok(M, na, nb);
+            const bool oz = ctx->g_tensor_cores && nmax > kCudaCoreG && g_ozaki_ok(M, na, nb);
             e = launch_gj<double>(ctx, Wk, P->C_alpha, P->C_beta, oz ? 0 : 1);
             if (e == cudaSuccess && oz) {
                 vmc_status st2 = launch_g_ozaki(ctx, Wk, P->C_alpha, P->C_beta, L->cdig);
@@ -990,11 +1033,11 @@ vmc_status launch_init_walkers(vmc_ctx *ctx, vmc_lists *L, const vmc_params *P, 
     if (e != cudaSuccess) return cuda_check(ctx, e, "k_init_tables");
     const double *js64 = (const double *)L->jsym;
     const float *js32 = (const float *)(js64 + 4 * (size_t)M * M);
-    const int sb = (Wk->W + kSumWalkers - 1) / kSumWalkers;
+    const int sb = (Wk->W + kSumWalkers - 1) / kSumWalkers, st_thr = std::max(1, VMC_THREADS / ((M + 31) / 32 * 32)) * ((M + 31) / 32 * 32);
     if (Wk->precision == VMC_FP64)
-        k_jastrow_sums<double><<<sb, VMC_THREADS, 0, ctx->stream>>>(Wk->W, M, js64, Wk->occ_bits, (double *)Wk->S);
+        k_jastrow_sums<double><<<sb, st_thr, 0, ctx->stream>>>(Wk->W, M, js64, Wk->occ_bits, (double *)Wk->S);
     else
-        k_jastrow_sums<float><<<sb, VMC_THREADS, 0, ctx->stream>>>(Wk->W, M, js32, Wk->occ_bits, (float *)Wk->S);
+        k_jastrow_sums<float><<<sb, st_thr, 0, ctx->stream>>>(Wk->W, M, js32, Wk->occ_bits, (float *)Wk->S);
     ctx->launches += 1;
     if (Wk->precision == VMC_MIXED && L->view.ns_pad > 0) {
         dim3 fg((unsigned)((L->view.ns_pad + kFockThreads - 1) / kFockThreads),
