@@ -36,9 +36,8 @@ __device__ __forceinline__ void weights(int mode, const double *t, const double 
 
 // Fixed-point weights for the Jastrow gradient: cq = round(c 2^s) with s chosen from sum |c| so that
 // no partial sum can overflow 63 bits; integer sums are then exact and order independent.
-// Also adds sum c0 and sum c1 to sums[0..1] (mode 1).  Three launches, each sum in a fixed order:
-// per-CTA partial sums over consecutive walker chunks, one warp that adds the partials and sets the
-// exponents, then the quantisation over the whole grid.
+// Also adds sum c0 and sum c1 to sums[0..1] (mode 1).  Two launches, each sum in a fixed order:
+// per-CTA partial sums over consecutive walker chunks, then the quantisation over the whole grid.
 constexpr int kWeightChunk = 256;   // walkers per partial-sum CTA
 constexpr int kWeightParts = 256;   // most partial sums (chunks grow beyond 65,536 walkers)
 
@@ -64,25 +63,32 @@ k_weight_partial(int W, int chunk, const double *__restrict__ t, const double *_
     }
 }
 
-__global__ void __launch_bounds__(32)
-k_weight_finish(int n_parts, const double *__restrict__ part, int *__restrict__ sexp, double *__restrict__ sums) {
-    double v[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int b = threadIdx.x; b < n_parts; b += 32)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) v[q] += part[(size_t)b * 4 + q];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) v[q] = warp_sum_f64(v[q]);
-    if (threadIdx.x == 0) {
-        sexp[0] = v[0] > 0.0 ? 61 - ilogb(v[0]) : 0;
-        sexp[1] = v[1] > 0.0 ? 61 - ilogb(v[1]) : 0;
-        if (sums) { sums[0] += v[2]; sums[1] += v[3]; }
-    }
-}
-
+// Adds the partials (one warp of every CTA, all in the same order, so that no launch of its own is needed for
+// it), sets the exponents and quantises; CTA 0 also stores the exponents and the sums.
 __global__ void __launch_bounds__(256)
-k_weight_quant(int W, const double *__restrict__ t, const double *__restrict__ e, int mode,
-               const int *__restrict__ sexp, long long *__restrict__ cq) {
-    const int e0 = sexp[0], e1 = sexp[1];
+k_weight_quant(int W, const double *__restrict__ t, const double *__restrict__ e, int mode, int n_parts,
+               const double *__restrict__ part, int *__restrict__ sexp, double *__restrict__ sums,
+               long long *__restrict__ cq) {
+    __shared__ int s_exp[2];
+    if (threadIdx.x < 32) {
+        double v[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int b = threadIdx.x; b < n_parts; b += 32)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v[q] += part[(size_t)b * 4 + q];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] = warp_sum_f64(v[q]);
+        if (threadIdx.x == 0) {
+            s_exp[0] = v[0] > 0.0 ? 61 - ilogb(v[0]) : 0;
+            s_exp[1] = v[1] > 0.0 ? 61 - ilogb(v[1]) : 0;
+            if (blockIdx.x == 0) {
+                sexp[0] = s_exp[0];
+                sexp[1] = s_exp[1];
+                if (sums) { sums[0] += v[2]; sums[1] += v[3]; }
+            }
+        }
+    }
+    __syncthreads();
+    const int e0 = s_exp[0], e1 = s_exp[1];
     for (int w = blockIdx.x * blockDim.x + threadIdx.x; w < W; w += gridDim.x * blockDim.x) {
         double c0, c1;
         weights(mode, t, e, w, c0, c1);
@@ -163,21 +169,31 @@ k_grad_J(int W, int M, const uint32_t *__restrict__ bits, const long long *__res
     }
 }
 
-__global__ void k_reduce_J(int M, int n_chunks, const long long *__restrict__ part, const int *__restrict__ sexp,
-                           double *__restrict__ dJ, double *__restrict__ dJ2) {
-    const int N2 = 2 * M;
+// Sum of the dJ partials over walker chunks (integers: any order).  CTA = 32 consecutive outputs (lanes) x 8 warps over
+// interleaved chunks: a small system has few outputs and as many chunks as the SMs leave it (H20: 76), which one
+// thread per output added one after the other (4,096 walkers: 11.9 -> 3.5 us).
+__global__ void __launch_bounds__(256)
+k_reduce_J(int M, int n_chunks, const long long *__restrict__ part, const int *__restrict__ sexp,
+           double *__restrict__ dJ, double *__restrict__ dJ2) {
+    __shared__ long long red[2][8][32];
+    const int N2 = 2 * M, lane = threadIdx.x & 31, v = threadIdx.x >> 5;
     const size_t csz = (size_t)N2 * N2;
-    const int e0 = sexp[0], e1 = sexp[1];
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < N2 * N2; t += gridDim.x * blockDim.x) {
-        const int p = t / N2, q = t % N2;
-        if (p > q) continue;
-        long long s = 0, s2 = 0;
-        for (int c = 0; c < n_chunks; ++c) s += part[(size_t)c * csz + t];
-        dJ[t] += scalbn((double)s, -e0);
-        if (dJ2) {
-            for (int c = 0; c < n_chunks; ++c) s2 += part[((size_t)n_chunks + c) * csz + t];
-            dJ2[t] += scalbn((double)s2, -e1);
+    const int t = blockIdx.x * 32 + lane, p = t / N2, q = t - p * N2;
+    const bool mine = t < N2 * N2 && p <= q;
+    long long s = 0, s2 = 0;
+    if (mine)
+        for (int c = v; c < n_chunks; c += 8) {
+            s += part[(size_t)c * csz + t];
+            if (dJ2) s2 += part[((size_t)n_chunks + c) * csz + t];
         }
+    red[0][v][lane] = s;
+    red[1][v][lane] = s2;
+    __syncthreads();
+    if (v < (dJ2 ? 2 : 1) && mine) {
+        long long sum = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) sum += red[v][k][lane];
+        (v ? dJ2 : dJ)[t] += scalbn((double)sum, -sexp[v]);
     }
 }
 
@@ -532,9 +548,9 @@ static vmc_status grad_impl(vmc_ctx *ctx, const vmc_walkers *Wk, const double *t
         const int wchunk = std::max(kWeightChunk, (W + kWeightParts - 1) / kWeightParts);
         const int n_parts = (W + wchunk - 1) / wchunk;
         k_weight_partial<<<n_parts, 256, 0, ctx->stream>>>(W, wchunk, t, e, mode, wpart);
-        k_weight_finish<<<1, 32, 0, ctx->stream>>>(n_parts, wpart, sexp, sums);
-        k_weight_quant<<<(W + 255) / 256 < 1216 ? (W + 255) / 256 : 1216, 256, 0, ctx->stream>>>(W, t, e, mode, sexp, cq);
-        ctx->launches += 3;
+        k_weight_quant<<<(W + 255) / 256 < 1216 ? (W + 255) / 256 : 1216, 256, 0, ctx->stream>>>(W, t, e, mode, n_parts, wpart,
+                                                                                                 sexp, sums, cq);
+        ctx->launches += 2;
     }
     if (out0[0]) {
         if (jtc) {
@@ -544,7 +560,7 @@ static vmc_status grad_impl(vmc_ctx *ctx, const vmc_walkers *Wk, const double *t
             k_grad_J<<<dim3(ntile, cj), 256, 0, ctx->stream>>>(W, M, Wk->occ_bits, cq, mode, (long long *)part);
             ctx->launches += 1;
         }
-        k_reduce_J<<<(N2 * N2 + 255) / 256, 256, 0, ctx->stream>>>(M, cj, (const long long *)part, sexp, out0[0],
+        k_reduce_J<<<(N2 * N2 + 31) / 32, 256, 0, ctx->stream>>>(M, cj, (const long long *)part, sexp, out0[0],
                                                                    mode ? out1[0] : nullptr);
         ctx->launches += 1;
         cudaError_t err = cudaGetLastError();
