@@ -171,7 +171,8 @@ k_grad_J(int W, int M, const uint32_t *__restrict__ bits, const long long *__res
 
 // Sum of the dJ partials over walker chunks (integers: any order).  CTA = 32 consecutive outputs (lanes) x 8 warps over
 // interleaved chunks: a small system has few outputs and as many chunks as the SMs leave it (H20: 76), which one
-// thread per output added one after the other (4,096 walkers: 11.9 -> 3.5 us).
+// thread per output added one after the other (4,096 walkers: 12.0 -> 4.0 us; H80, 16,384 walkers: 7.3 -> 3.4 us; H160,
+// 32,768 walkers, where outputs are many: 5.6 -> 6.1 us).
 __global__ void __launch_bounds__(256)
 k_reduce_J(int M, int n_chunks, const long long *__restrict__ part, const int *__restrict__ sexp,
            double *__restrict__ dJ, double *__restrict__ dJ2) {

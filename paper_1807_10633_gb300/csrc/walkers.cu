@@ -902,7 +902,7 @@ k_log_psi(int M, int na, int nb, const double *__restrict__ Ca, const double *__
 // unused row with the largest |a_k| (keys compared as integers; NaN lowest, ties to the lowest row) is
 // broadcast element by element and eliminated from the other unused rows.  At these sizes the CTA-wide
 // elimination is barriers and latency: 4,096 walkers of H40 took 952 us with it (one FP64 division and an
-// integer division per updated element), 130 us with this kernel.
+// integer division per updated element), 244 us with this kernel (its n^3 / 3 multiply-adds alone: about 40 us; the rest is the serial chain of pivots).
 constexpr int kLogWarps = 8;     // four walkers per CTA
 
 template <int NP>
