@@ -2,18 +2,18 @@
 //
 // One CTA per walker.  The walker's G (virtual rows only), exp(S) and the orbital -> column /
 // slot map are staged in shared memory; the screened lists (shared by all walkers, L2-resident)
-// are streamed per occupied pair.  Work is split into "groups" in canonical move order:
-//   singles : blocks of 32 consecutive spin orbitals i; unit = occupied i, list = singles(i)
-//   doubles : one group per alpha spin-orbital row i (warp chunks of 32 candidates if needed);
-//             the candidates j > i of a row are the spin orbitals whose spatial index lies within
-//             the band of non-empty pair lists (same spin: q in (p, p+B]; alpha rows also
-//             opposite spin q in [p-B, p+B]), so a row fits one warp for local orbitals.  Beta
-//             rows have only the B same-spin candidates; floor(32 / B) of them share a group.
-// A warp takes one group; its active units (i and j occupied, list non-empty) are walked in
-// order with the lanes over each unit's list entries.  Each group's CTMC rates are summed as
-// exact 128-bit fixed-point integers (order independent) and stored; the CTMC kernel re-walks
-// only the chosen group.  Every product that enters a rate uses explicitly rounded intrinsics
-// so the two kernels compute bit-identical rates.
+// are one flat array of entries in canonical move order, each with its orbitals (i, j, a, b).
+// Which entries are moves is a row of bits per walker (i, j occupied, a, b empty, above eps_run),
+// made for 64 walkers at once by k_free_bits, or by the walker's own CTA when the row is short.
+// Entries belong to "groups":
+//   singles : blocks of 32 consecutive spin orbitals i
+//   doubles : one group per alpha spin-orbital row i (parts of it if needed); beta rows, which have
+//             only the same-spin candidates, share groups.
+// A warp takes a group, compacts the set bits of its part of the row and evaluates 32 moves at a
+// time.  Each group's CTMC rates are summed as exact 128-bit fixed-point integers (order
+// independent) and stored; the CTMC kernel re-walks only the chosen group, from the same bits.
+// Every product that enters a rate uses explicitly rounded intrinsics so the two kernels compute
+// bit-identical rates.  k_screened_moves walks the lists unit by unit (setup_unit), without the bits.
 #include <math.h>
 
 #include <algorithm>
