@@ -150,14 +150,15 @@ class Clocks:
                 "reasons": sorted(reasons), "samples": len(sm)}
 
 
-# ncu counters of one k_local_energy launch (mixed form, H160, eps 1e-6, 4,096 walkers), per walker:
+# ncu counters of one local energy, k_free_bits and k_local_energy together (mixed form, H160, eps 1e-6,
+# 4,096 walkers), per walker:
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum), L2 bytes (lts__t_sectors.sum x 32) and
 # warp instructions (smsp__inst_executed.sum), from the capture summarised in
 # profiles/k_local_energy_mixed_h160_w4096.md.  They describe the kernel source with this digest
 # only; any later change of the kernel's file reports traffic as null until it is captured again.
-ELOC_COUNTERS = {"sha256": "2ce2119c06f96ce3069d3b8429e711f38fb44c503e99b0be541f82c9f7cb0725",
-                 "system": "H160", "eps": 1e-6, "dram_bytes_per_walker": 80584.9, "l2_bytes_per_walker": 875568.0,
-                 "warp_inst_per_walker": 219949.0}
+ELOC_COUNTERS = {"sha256": "60394967b2157dd5532e1a73589eb86585ed0fcf87f153270902cfbbe68aab2c",
+                 "system": "H160", "eps": 1e-6, "dram_bytes_per_walker": 119893.3, "l2_bytes_per_walker": 759253.3,
+                 "warp_inst_per_walker": 173000.4}
 
 
 def counters_apply(system: str, eps: float) -> bool:
