@@ -136,6 +136,9 @@ vmc_status vmc_screened_lists_summary(int M, const double *h_h1, const double *h
  *                     (i -> a) and spin (the elements of Sec. II.A, kept up to date per move;
  *                     ns_pad = n_singles rounded up to a multiple of 4, padding entries zero;
  *                     the mixed form recomputes them at every refresh)
+ *                     Must start on a 16-byte boundary for the moves (vmc_ctmc_step and
+ *                     vmc_ctmc_step_batch return VMC_ERR_ARG otherwise); the other arrays only
+ *                     need the alignment of their elements.
  *   e_diag    double [W]       <n|H|n> including e_core
  *   rng_counter uint64 [W]     Philox counter of each walker (advanced by vmc_ctmc_step)
  * real = double for VMC_FP64, float for VMC_MIXED.  The orbital order inside occ_list and

@@ -53,6 +53,12 @@ static vmc_status check_walkers(vmc_ctx *ctx, const vmc_walkers *Wk, const vmc_l
     return VMC_OK;
 }
 
+// The move update reads and writes the Fock sums as 16-byte vectors.
+static vmc_status check_fock(vmc_ctx *ctx, const vmc_walkers *Wk, const vmc_lists *L) {
+    if (L->ns > 0 && (uintptr_t)Wk->F % 16) return set_err(ctx, VMC_ERR_ARG, "F must start on a 16-byte boundary");
+    return VMC_OK;
+}
+
 extern "C" {
 
 vmc_status vmc_create(vmc_ctx **out, int device, void *stream) {
@@ -201,6 +207,8 @@ vmc_status vmc_ctmc_step(vmc_ctx *ctx, const vmc_lists *L, const vmc_params *P, 
     if (!L || !P || !P->J || !move_code) return set_err(ctx, VMC_ERR_ARG, "null argument");
     vmc_status st = check_walkers(ctx, Wk, L);
     if (st) return st;
+    st = check_fock(ctx, Wk, L);
+    if (st) return st;
     if (!ctx->rates_valid || ctx->rates_walkers != Wk->G)
         return set_err(ctx, VMC_ERR_ARG, "vmc_local_energy must precede vmc_ctmc_step on the same walkers");
     st = check_cps(ctx, P, Wk);
@@ -248,6 +256,8 @@ vmc_status vmc_ctmc_step_batch(vmc_ctx *ctx, int n, const vmc_batch_item *items,
         if (st) return st;
         if (items[k].params && items[k].params->cps)
             return set_err(ctx, VMC_ERR_ARG, "the batched launches do not take a correlator product");
+        if (items[k].lists) st = check_fock(ctx, items[k].walkers, items[k].lists);
+        if (st) return st;
     }
     return launch_ctmc_step_batch(ctx, n, items, seed);
 }

@@ -319,8 +319,8 @@ k_grad_C_reg(int W, int M, int na, int nb, const uint16_t *__restrict__ pos, con
     const size_t aoff = s ? (size_t)na * na : 0;
     const int w0 = blockIdx.y * kChunkC, w1 = min(W, w0 + kChunkC);
     const bool xin = x < n;
-    // the kRowsC map entries of a walker: two 16-byte loads when aligned (M % 8 == 0)
-    const bool vec = (M & 7) == 0 && k0 + kRowsC <= M;
+    // the kRowsC map entries of a walker: two 16-byte loads when aligned (M % 8 == 0 and the caller's array)
+    const bool vec = (M & 7) == 0 && k0 + kRowsC <= M && (uintptr_t)pos % 16 == 0;
     auto map_of = [&](int w, uint4 &lo, uint4 &hi) {
         const uint16_t *pw = pos + (size_t)w * 2 * M + (size_t)s * M + k0;
         if (vec) {

@@ -751,6 +751,7 @@ k_jastrow_sums(int W, int M, const real *__restrict__ Jsym, const uint32_t *__re
     }
     __syncthreads();
     const real2 *J2 = (const real2 *)Jsym;               // rows of M pairs
+    const bool pairs = (uintptr_t)S % sizeof(real2) == 0;     // the caller's array: as any of its elements may be
     const int per = (M + 31) / 32 * 32, groups = max(1, (int)blockDim.x / per);    // threads of a walker, walkers at a time
     const int grp = threadIdx.x / per;
     for (int h = threadIdx.x - grp * per; h < M && grp < groups; h += per) {
@@ -786,7 +787,12 @@ k_jastrow_sums(int W, int M, const real *__restrict__ Jsym, const uint32_t *__re
             real2 out;
             out.x = occ(p) ? acc0 - jd0 : acc0;
             out.y = occ(p + 1) ? acc1 - jd1 : acc1;
-            ((real2 *)S)[(size_t)(w0 + k) * M + h] = out;
+            if (pairs) {
+                ((real2 *)S)[(size_t)(w0 + k) * M + h] = out;
+            } else {
+                S[(size_t)(w0 + k) * N2 + p] = out.x;
+                S[(size_t)(w0 + k) * N2 + p + 1] = out.y;
+            }
         }
     }
 }

@@ -1,0 +1,56 @@
+"""Host side of the library's calls on a CUDA runtime without a device (CPU only): what is refused before a launch,
+what the context's rate store holds, and when it is allocated."""
+import pytest
+
+from paper_1807_10633_gb300 import systems as S
+from paper_1807_10633_gb300 import vmc
+from tests import fake_cudart
+
+
+@pytest.fixture(scope="module")
+def runtime(tmp_path_factory):
+    path = fake_cudart.build(tmp_path_factory.mktemp("fake"))
+    keep = vmc.LIB, vmc._lib
+    vmc.LIB, vmc._lib = path, None
+    yield fake_cudart.Runtime(vmc.lib())
+    vmc.LIB, vmc._lib = keep
+
+
+@pytest.fixture
+def ctx(runtime):
+    runtime.limit()
+    c = vmc.vmc_create(0, 0)
+    runtime.launches()
+    yield c
+    runtime.limit()
+    vmc.vmc_destroy(c)
+
+
+def _refused(call, *args, **kw):
+    with pytest.raises(vmc.VmcError) as e:
+        call(*args, **kw)
+    assert e.value.status == 1, e.value                  # VMC_ERR_ARG
+    return str(e.value)
+
+
+@pytest.mark.parametrize("precision,shift", [(0, 8), (1, 4), (1, 8)])
+def test_moves_need_aligned_fock_sums(runtime, ctx, precision, shift):
+    """The update reads F as 16-byte vectors: a misaligned F is refused before any kernel, alone and in a batch; the
+    other arrays may start at any of their elements."""
+    sys_ = S.named_system("H6")
+    bad = fake_cudart.System(ctx, sys_, 5, 1e-6, precision, {"F": shift})
+    bad.energy()
+    runtime.launches()
+    assert "16-byte" in _refused(bad.step)
+    items = fake_cudart.batch([bad])
+    vmc.vmc_local_energy_batch(ctx, items)
+    runtime.launches()
+    assert "16-byte" in _refused(vmc.vmc_ctmc_step_batch, ctx, items, 3)
+    assert runtime.launches() == []
+    real = 8 if precision == 0 else 4
+    ok = fake_cudart.System(ctx, sys_, 5, 1e-6, precision, {"S": real, "G": real, "AinvT": real, "pos": 2, "occ_list": 2})
+    ok.energy()
+    ok.step()
+    assert any("k_ctmc_apply" in x for x in runtime.launches())
+    for s in (bad, ok):
+        s.close()
