@@ -246,7 +246,7 @@ vmc_status vmc_local_energy(vmc_ctx *ctx, const vmc_lists *lists, const vmc_para
 /*
  * Continuous-time Monte Carlo move (Sec. II.B): for every walker pick the next determinant with
  * probability proportional to its rate, without rejection, from the rates stored by the last
- * vmc_local_energy on the same walkers (which must come first: VMC_ERR_ARG otherwise), then
+ * vmc_local_energy on the same walkers and lists (which must come first: VMC_ERR_ARG otherwise), then
  * update the walker in O(N^2): Sherman-Morrison (rank-1, or rank-2 Woodbury for same-spin
  * doubles) on G and AinvT, Jastrow sums, Fock sums, e_diag, bits and lists.
  * Choice rule: q_k = floor(r_k 2^64) (exact 128-bit), U = word 0 of

@@ -6,8 +6,6 @@
 
 #include "common.cuh"
 
-vmc_status lists_set_eps(vmc_ctx *ctx, vmc_lists *L, double eps_run);
-
 vmc_status set_err(vmc_ctx *ctx, vmc_status st, const std::string &msg) {
     if (ctx) ctx->err = msg;
     return st;
@@ -192,11 +190,9 @@ vmc_status vmc_local_energy(vmc_ctx *ctx, const vmc_lists *Lc, const vmc_params 
     if (st) return st;
     st = lists_set_eps(ctx, L, eps_run);
     if (st) return st;
-    const int ng = L->view.n_groups;
     st = launch_local_energy(ctx, L, Wk, cps_view(P), e_loc, t_res);
     if (st) return st;
-    ctx->rates_walkers = Wk->G;
-    ctx->rates_groups = ng;
+    ctx->rates_of = StoredRates{Wk->G, Wk->W, L->view.n_groups, L->view.words, L->digest, eps_run};
     ctx->rates_valid = 1;
     return VMC_OK;
 }
@@ -209,11 +205,15 @@ vmc_status vmc_ctmc_step(vmc_ctx *ctx, const vmc_lists *L, const vmc_params *P, 
     if (st) return st;
     st = check_fock(ctx, Wk, L);
     if (st) return st;
-    if (!ctx->rates_valid || ctx->rates_walkers != Wk->G)
+    const StoredRates &r = ctx->rates_of;
+    if (!ctx->rates_valid || r.G != Wk->G || Wk->W > r.W)
         return set_err(ctx, VMC_ERR_ARG, "vmc_local_energy must precede vmc_ctmc_step on the same walkers");
+    if (!same_lists(r, L)) return set_err(ctx, VMC_ERR_ARG, "vmc_ctmc_step on other lists than vmc_local_energy");
     st = check_cps(ctx, P, Wk);
     if (st) return st;
-    st = launch_ctmc_step(ctx, L, P, Wk, seed, (const u128 *)ctx->rates, ctx->rates_groups, move_code);
+    st = lists_set_eps(ctx, const_cast<vmc_lists *>(L), r.eps);   // (another context may have run them at its own)
+    if (st) return st;
+    st = launch_ctmc_step(ctx, L, P, Wk, seed, move_code);
     ctx->rates_valid = 0;
     return st;
 }

@@ -21,6 +21,15 @@ typedef unsigned __int128 u128;
 #define VMC_DEV_INCONSISTENT 8u
 #define VMC_DEV_TIMEOUT 16u
 
+// What one system's part of the rate store was computed from.  Rates and free-entry rows are laid out by the
+// lists, so the moves may read them with the same lists alone (by content) and with no more walkers.
+struct StoredRates {
+    const void *G = nullptr;     // of the walkers
+    int W = 0, n_groups = 0, words = 0;
+    uint64_t lists = 0;          // vmc_lists::digest
+    double eps = 0.0;            // eps_run
+};
+
 struct vmc_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
@@ -35,9 +44,8 @@ struct vmc_ctx {
     void *bits = nullptr;        // in rates: the free-entry rows of the last vmc_local_energy's walkers
     int bits_whole = 0;          // they hold every walker of the last vmc_local_energy
     // rate store bookkeeping (vmc_local_energy -> vmc_ctmc_step)
-    const void *rates_walkers = nullptr;
+    StoredRates rates_of;
     int rates_valid = 0;
-    int rates_groups = 0;
     uint64_t launches = 0;
     // batched launches: device descriptor table (re-uploaded only when the batch changes)
     void *batch_desc = nullptr;
@@ -126,6 +134,7 @@ struct vmc_lists {
     int M = 0;
     double eps_build = 0.0;
     double eps_run = -1.0;   // eps the effective lengths were computed for
+    uint64_t digest = 0;     // of the moves and their magnitudes, in canonical order
     int64_t near_ties_build = 0;   // near ties of the build eps over every candidate (Sec. II.A)
     int64_t ns = 0, nds = 0, ndo = 0;
     // host copies of the sorted magnitudes (for effective lengths at a given eps_run)
@@ -141,6 +150,10 @@ struct vmc_lists {
     const double *jastrow_for = nullptr;   // J pointer the constants were refreshed for
     uint64_t jastrow_epoch = 0;
 };
+
+inline bool same_lists(const StoredRates &r, const vmc_lists *L) {
+    return r.lists == L->digest && r.n_groups == L->view.n_groups && r.words == L->view.words;
+}
 
 // ------------------------------------------------------------------ small helpers
 __host__ __device__ inline int tri_index(int p, int q, int M) {  // p < q
@@ -261,6 +274,7 @@ cudaError_t launch_dependent(bool dependent, void (*kernel)(KArgs...), dim3 grid
 vmc_status set_err(vmc_ctx *ctx, vmc_status st, const std::string &msg);
 vmc_status cuda_check(vmc_ctx *ctx, cudaError_t e, const char *what);
 vmc_status ensure_workspace(vmc_ctx *ctx, size_t bytes);
+vmc_status lists_set_eps(vmc_ctx *ctx, vmc_lists *L, double eps_run);
 size_t walker_stride_G(int M, int na, int nb);
 size_t walker_stride_A(int na, int nb);
 
@@ -272,8 +286,7 @@ struct CpsView;
 vmc_status launch_local_energy(vmc_ctx *ctx, const vmc_lists *L, vmc_walkers *Wk, const CpsView &C,
                                double *e_loc, double *t_res);
 vmc_status launch_ctmc_step(vmc_ctx *ctx, const vmc_lists *L, const vmc_params *P,
-                            vmc_walkers *Wk, uint64_t seed, const u128 *rates, int n_groups,
-                            uint64_t *move_code);
+                            vmc_walkers *Wk, uint64_t seed, uint64_t *move_code);
 vmc_status launch_screened_moves(vmc_ctx *ctx, const vmc_lists *L, const vmc_walkers *Wk, const CpsView &C,
                                  int w_begin, int n_w, int64_t cap, uint64_t *code, double *ratio, double *contrib,
                                  int64_t *count, int64_t *walked);

@@ -1646,9 +1646,9 @@ static cudaError_t ctmc_launch(vmc_ctx *ctx, const vmc_lists *L, const vmc_param
 }
 
 vmc_status launch_ctmc_step(vmc_ctx *ctx, const vmc_lists *L, const vmc_params *P, vmc_walkers *Wk,
-                            uint64_t seed, const u128 *rates, int n_groups, uint64_t *move_code) {
+                            uint64_t seed, uint64_t *move_code) {
     const int M = Wk->M;
-    (void)n_groups;
+    const u128 *rates = (const u128 *)ctx->rates;
     const int nmax = Wk->n_alpha > Wk->n_beta ? Wk->n_alpha : Wk->n_beta;
     const size_t esz = Wk->precision == VMC_FP64 ? 8 : 4;
     const size_t smem = 2 * (2 * (size_t)M) + 32 + esz * (4 * (size_t)((nmax + 3) & ~3) + 2 * (size_t)((M + 3) & ~3));
@@ -1688,7 +1688,6 @@ struct BatchPlan {
 // then one per round of the local energy.  Also sizes the shared rate store and the free-entry rows:
 // every system's walkers are split over as few rounds as keep the rows within kBitsCap.
 static vmc_status prepare_batch(vmc_ctx *ctx, int n, const vmc_batch_item *items, BatchPlan &plan) {
-    extern vmc_status lists_set_eps(vmc_ctx *, vmc_lists *, double);
     if (n < 1 || n > 64 || !items) return set_err(ctx, VMC_ERR_ARG, "1 to 64 batch items");
     std::vector<int> order(n);
     std::vector<double> cost(n);

@@ -228,6 +228,17 @@ template <typename T> void digest_add(uint64_t &h, const std::vector<T> &v) {
     }
 }
 
+// The same over 64-bit words: a digest of the lists that a build can afford
+void digest_words(uint64_t &h, const void *p, size_t bytes) {
+    const unsigned char *b = (const unsigned char *)p;
+    for (size_t k = 0; k < bytes; k += 8) {
+        uint64_t x = 0;
+        memcpy(&x, b + k, std::min<size_t>(8, bytes - k));
+        h = (h ^ x) * 0x9E3779B97F4A7C15ull;
+        h ^= h >> 29;
+    }
+}
+
 const char *check_build_args(int M, const double *h1, const double *eri, int eri_packed, double eps) {
     if (!h1 || !eri) return "null argument";
     if (M < 1 || M > VMC_MAX_M) return "M must be in [1, 256]";
@@ -460,6 +471,12 @@ extern "C" vmc_status vmc_build_screened_lists(vmc_ctx *ctx, int M, const double
     }
     v.words = (int)(F.key.size() / 32);
     L->h_base = dup_u32(F.base);
+    digest_words(L->digest, F.base.data(), sizeof(uint32_t) * F.base.size());
+    digest_words(L->digest, F.key.data(), sizeof(uint32_t) * F.key.size());
+    digest_words(L->digest, F.wcls.data(), F.wcls.size());
+    digest_words(L->digest, H.s_key.data(), sizeof(double) * H.s_key.size());
+    digest_words(L->digest, H.ds_key.data(), sizeof(double) * H.ds_key.size());
+    digest_words(L->digest, H.do_key.data(), sizeof(double) * H.do_key.size());
     // scaling costs two products for each of about M^2 / 2 elements of G and saves four per free double; about
     // one entry in eight is free.  (8 x 8 Hubbard lattice, singles alone: 68 us without, 86 us with it for
     // 4,000 walkers; H160 at 1e-6: 13.2 -> 11.5 ms with it for 32,768.)

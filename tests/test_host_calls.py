@@ -54,3 +54,36 @@ def test_moves_need_aligned_fock_sums(runtime, ctx, precision, shift):
     assert any("k_ctmc_apply" in x for x in runtime.launches())
     for s in (bad, ok):
         s.close()
+
+
+def test_moves_refuse_rates_of_other_lists(runtime, ctx):
+    """Rates and rows are laid out by the lists of the local energy: other lists of the same size, or more walkers than
+    it had, are refused; a second build of the same lists is the same lists."""
+    s = fake_cudart.System(ctx, S.named_system("H12"), 700, 1e-4)
+    same = fake_cudart.System(ctx, S.named_system("H12"), 1, 1e-4)
+    other = fake_cudart.System(ctx, S.named_system("H12"), 1, 1e-6)
+    s.energy()
+    runtime.launches()
+    assert "lists" in _refused(s.step, other.lists)
+    s.walkers.W = 701
+    assert "walkers" in _refused(s.step)
+    assert runtime.launches() == []
+    s.walkers.W = 700
+    s.step(same.lists)
+    assert any("k_ctmc_select" in x for x in runtime.launches())
+    for x in (s, same, other):
+        x.close()
+
+
+def test_moves_use_the_threshold_of_their_rates(runtime, ctx):
+    """Another context may run the same lists at another eps_run in between: the choice is made at the rates' own."""
+    s = fake_cudart.System(ctx, S.named_system("H12"), 700, 1e-6)
+    c2 = vmc.vmc_create(0, 0)
+    s.energy(1e-5)
+    s.energy(1e-3, c2)
+    s.step()
+    before = runtime.counts()["uploads"]
+    s.energy(1e-5)                                       # the lists stand at 1e-5 again: nothing to upload
+    assert runtime.counts()["uploads"] == before
+    vmc.vmc_destroy(c2)
+    s.close()
