@@ -292,7 +292,8 @@ vmc_status vmc_screened_moves(vmc_ctx *ctx, const vmc_lists *lists, const vmc_pa
  * vmc_ctmc_step_batch then moves every walker (selection and update, one launch each).  Results
  * are identical to the per-system calls (walker index and seed as in vmc_ctmc_step).  The first
  * call with a new set of items uploads a small descriptor table (not capturable); later calls with
- * the same items are.  vmc_ctmc_step_batch must follow vmc_local_energy_batch on the same items.
+ * the same items are.  vmc_ctmc_step_batch must follow vmc_local_energy_batch on the same items, with no
+ * local energy, initialisation or refresh on this context in between (VMC_ERR_ARG otherwise).
  */
 typedef struct {
     const vmc_lists *lists;

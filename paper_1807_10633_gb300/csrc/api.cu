@@ -164,7 +164,7 @@ static vmc_status init_common(vmc_ctx *ctx, vmc_lists *L, const vmc_params *P, v
     if (st) return st;
     st = check_cps(ctx, P, Wk);
     if (st) return st;
-    ctx->rates_valid = 0;
+    drop_rates(ctx);
     st = launch_init_walkers(ctx, L, P, Wk, full);
     if (st) return st;
     return launch_cps_state(ctx, P, Wk);

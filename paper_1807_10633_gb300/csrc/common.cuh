@@ -151,6 +151,12 @@ struct vmc_lists {
     uint64_t jastrow_epoch = 0;
 };
 
+// The rate store is about to change, or the tables that its rates belong to.
+inline void drop_rates(vmc_ctx *ctx) {
+    ctx->rates_valid = 0;
+    ctx->rates_batch.clear();
+}
+
 inline bool same_lists(const StoredRates &r, const vmc_lists *L) {
     return r.lists == L->digest && r.n_groups == L->view.n_groups && r.words == L->view.words;
 }

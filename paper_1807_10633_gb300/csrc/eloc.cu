@@ -1557,8 +1557,7 @@ static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Frees the store and allocates `bytes`; a failed allocation leaves none.
 static cudaError_t grow_store(vmc_ctx *ctx, size_t bytes) {
-    ctx->rates_valid = 0;
-    ctx->rates_batch.clear();
+    drop_rates(ctx);
     if (ctx->rates) {
         const cudaError_t e = cudaStreamSynchronize(ctx->stream);
         if (e != cudaSuccess) return e;
@@ -1608,6 +1607,7 @@ vmc_status launch_local_energy(vmc_ctx *ctx, const vmc_lists *L, vmc_walkers *Wk
     if (!eloc_fits(Wk, C, ctx->eloc_threads)) return set_err(ctx, VMC_ERR_ARG, "walker G table does not fit in shared memory");
     WalkerArgs A = make_args(Wk);
     const bool own = own_rows(L->view.words, Wk->W);
+    drop_rates(ctx);
     ctx->bits_whole = 0;
     int chunk = Wk->W;
     const size_t rates_bytes = sizeof(u128) * rate_store_units(Wk->W, L->view.n_groups);
@@ -1628,7 +1628,7 @@ vmc_status launch_local_energy(vmc_ctx *ctx, const vmc_lists *L, vmc_walkers *Wk
         ctx->launches += 1;
         if (e == cudaSuccess) e = cudaGetLastError();
     }
-    ctx->bits_whole = !own && chunk >= Wk->W;      // for the choice of the next move
+    ctx->bits_whole = e == cudaSuccess && !own && chunk >= Wk->W;      // for the choice of the next move
     return cuda_check(ctx, e, "k_local_energy");
 }
 
@@ -1818,6 +1818,7 @@ vmc_status launch_local_energy_batch(vmc_ctx *ctx, int n, const vmc_batch_item *
     int dev = 0, nsm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    drop_rates(ctx);
     for (int r = 0; r < plan.rounds && e == cudaSuccess; ++r) {
         const SysDesc *tab = (const SysDesc *)ctx->batch_desc + (plan.rounds > 1 ? (size_t)(r + 1) * n : 0);
         const int total = plan.walkers[r], tiles = plan.tiles[r];
@@ -1832,7 +1833,6 @@ vmc_status launch_local_energy_batch(vmc_ctx *ctx, int n, const vmc_batch_item *
     }
     if (e != cudaSuccess) return cuda_check(ctx, e, "k_local_energy_batched");
     ctx->rates_batch = batch_signature(n, items);
-    ctx->rates_valid = 0;
     return VMC_OK;
 }
 

@@ -87,3 +87,28 @@ def test_moves_use_the_threshold_of_their_rates(runtime, ctx):
     assert runtime.counts()["uploads"] == before
     vmc.vmc_destroy(c2)
     s.close()
+
+
+def _two(ctx, W=700):
+    return [fake_cudart.System(ctx, S.named_system("H12"), W, 1e-6), fake_cudart.System(ctx, S.named_system("H6"), 40, 1e-6)]
+
+
+@pytest.mark.parametrize("between", ["energy", "refresh", "init"])
+def test_batched_moves_need_their_own_energies(runtime, ctx, between):
+    """A local energy or a rebuild of the tables on the context takes the batch's rates with it, as it does those of a
+    single system."""
+    two = _two(ctx)
+    items = fake_cudart.batch(two)
+    vmc.vmc_local_energy_batch(ctx, items)
+    if between == "energy":
+        two[1].energy()
+    else:
+        call = vmc.vmc_walkers_refresh if between == "refresh" else vmc.vmc_walkers_init
+        call(ctx, two[0].lists, two[0].params, two[0].walkers)
+    runtime.launches()
+    assert "must precede" in _refused(vmc.vmc_ctmc_step_batch, ctx, items, 3)
+    assert runtime.launches() == []
+    vmc.vmc_local_energy_batch(ctx, items)
+    vmc.vmc_ctmc_step_batch(ctx, items, 3)
+    for s in two:
+        s.close()
