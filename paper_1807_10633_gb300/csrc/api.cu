@@ -294,7 +294,7 @@ vmc_status vmc_autotune_local_energy(vmc_ctx *ctx, int n, const vmc_batch_item *
     cudaEventDestroy(a);
     cudaEventDestroy(b);
     ctx->eloc_threads = pick;
-    ctx->rates_batch.clear();
+    ctx->batch_parts.clear();
     if (threads_out) *threads_out = pick;
     return VMC_OK;
 }

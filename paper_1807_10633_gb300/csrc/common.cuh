@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <string>
+#include <vector>
 
 #include "vmc.h"
 
@@ -30,6 +31,12 @@ struct StoredRates {
     double eps = 0.0;            // eps_run
 };
 
+// One item of a batched local energy: its rates, and where they and its rows stand in the store.
+struct BatchPart : StoredRates {
+    size_t rates_at = 0, bits_at = 0;    // 16-byte units; bytes
+    int share = 0;                       // walkers per round
+};
+
 struct vmc_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
@@ -52,7 +59,8 @@ struct vmc_ctx {
     size_t batch_desc_bytes = 0;
     std::string batch_host;
     int *d_queue = nullptr;
-    std::string rates_batch;       // walker tables the batched rate store belongs to
+    std::vector<BatchPart> batch_parts;   // vmc_local_energy_batch -> vmc_ctmc_step_batch, by item (none: not valid)
+    int batch_rounds = 1;
     int eloc_threads = 256;        // threads per local-energy CTA (set by the autotuner)
     int g_tensor_cores = 1;        // refresh: G on tcgen05 (1) or CUDA cores (0)
     int refresh_smem = 0;          // refresh: register Gauss-Jordan (0) or shared-memory LU/GJ (1)
@@ -154,7 +162,7 @@ struct vmc_lists {
 // The rate store is about to change, or the tables that its rates belong to.
 inline void drop_rates(vmc_ctx *ctx) {
     ctx->rates_valid = 0;
-    ctx->rates_batch.clear();
+    ctx->batch_parts.clear();
 }
 
 inline bool same_lists(const StoredRates &r, const vmc_lists *L) {

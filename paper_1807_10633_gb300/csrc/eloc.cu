@@ -1681,13 +1681,48 @@ struct BatchPlan {
     size_t smem_eloc = 0, smem_apply = 0;
     std::vector<int> walkers, tiles;   // per round
     int words = 0;                     // the longest free-entry row
+    std::vector<BatchPart> parts;      // the store's layout, by item
 };
+
+// The layout of a batch's rate store: every system's rates, then, for as many walkers as a round takes, its
+// free-entry rows.  The rounds are doubled until they fit.
+static vmc_status place_batch(vmc_ctx *ctx, int n, const vmc_batch_item *items, const std::vector<int> &order, BatchPlan &plan) {
+    plan.parts.assign(n, BatchPart());
+    size_t units = 0;
+    for (int k : order) {
+        const vmc_batch_item &it = items[k];
+        const ListsView &v = it.lists->view;
+        static_cast<StoredRates &>(plan.parts[k]) =
+            StoredRates{it.walkers->G, it.walkers->W, v.n_groups, v.words, it.lists->digest, it.eps_run};
+        plan.parts[k].rates_at = units;
+        units += rate_store_units(it.walkers->W, v.n_groups);
+    }
+    const size_t bits_at = align256(units * sizeof(u128));
+    for (plan.rounds = 1;; plan.rounds *= 2) {
+        size_t at = bits_at;
+        bool more = false;
+        for (int k : order) {
+            BatchPart &p = plan.parts[k];
+            p.share = ((p.W + plan.rounds - 1) / plan.rounds + 31) & ~31;
+            more = more || p.share > 32;
+            p.bits_at = at;
+            at += row_bytes(items[k].lists->view) * (size_t)p.share;
+        }
+        const size_t bytes = at + 32;
+        if (bytes <= ctx->rates_bytes) return VMC_OK;
+        if (bytes - bits_at > kBitsCap && more) continue;
+        const cudaError_t e = grow_store(ctx, bytes);
+        if (e == cudaSuccess) return VMC_OK;
+        if (e != cudaErrorMemoryAllocation || !more) return cuda_check(ctx, e, "batched rate store");
+    }
+}
 
 // Builds (and uploads when changed) the descriptor tables of a batch, most expensive systems first:
 // one table over all walkers (used by the CTMC step, and by the local energy when one round is enough),
-// then one per round of the local energy.  Also sizes the shared rate store and the free-entry rows:
-// every system's walkers are split over as few rounds as keep the rows within kBitsCap.
-static vmc_status prepare_batch(vmc_ctx *ctx, int n, const vmc_batch_item *items, BatchPlan &plan) {
+// then one per round of the local energy.  For the local energy (step = false) it also sizes the shared
+// rate store and the free-entry rows: every system's walkers are split over as few rounds as keep the rows within
+// kBitsCap.  The CTMC step reads the store as the local energy laid it out, and never resizes it.
+static vmc_status prepare_batch(vmc_ctx *ctx, int n, const vmc_batch_item *items, bool step, BatchPlan &plan) {
     if (n < 1 || n > 64 || !items) return set_err(ctx, VMC_ERR_ARG, "1 to 64 batch items");
     std::vector<int> order(n);
     std::vector<double> cost(n);
@@ -1699,7 +1734,7 @@ static vmc_status prepare_batch(vmc_ctx *ctx, int n, const vmc_batch_item *items
             return set_err(ctx, VMC_ERR_ARG, "batch items must share the precision");
         if (it.walkers->M != it.lists->M) return set_err(ctx, VMC_ERR_ARG, "lists and walkers disagree on M");
         if (!(it.eps_run >= it.lists->eps_build)) return set_err(ctx, VMC_ERR_ARG, "eps_run below the build eps");
-        vmc_status st = lists_set_eps(ctx, const_cast<vmc_lists *>(it.lists), it.eps_run);
+        vmc_status st = lists_set_eps(ctx, const_cast<vmc_lists *>(it.lists), step ? ctx->batch_parts[k].eps : it.eps_run);
         if (st) return st;
         order[k] = k;
         const vmc_lists *L = it.lists;
@@ -1707,49 +1742,32 @@ static vmc_status prepare_batch(vmc_ctx *ctx, int n, const vmc_batch_item *items
                   (double)walker_stride_G(it.walkers->M, it.walkers->n_alpha, it.walkers->n_beta);
     }
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cost[a] > cost[b]; });
-    size_t rates_total = 0;
-    std::vector<size_t> rate_off(n);
     int tot = 0;
     size_t se = 0, sa = 0;
     for (int k = 0; k < n; ++k) {
         const vmc_batch_item &it = items[order[k]];
-        rate_off[k] = rates_total;
-        rates_total += rate_store_units(it.walkers->W, it.lists->view.n_groups);
         tot += it.walkers->W;
         se = std::max(se, eloc_smem_bytes(it.lists->view, it.walkers, CpsView{}, ctx->eloc_threads));
         plan.fits = plan.fits && eloc_fits(it.walkers, CpsView{}, ctx->eloc_threads);
         sa = std::max(sa, apply_smem_bytes(it.walkers));
     }
-    // free-entry rows: rounds (doubled) until every system's share fits
-    const size_t bits_at = align256(rates_total * sizeof(u128));
-    std::vector<int> share(n);
-    int rounds = 1;
-    for (;; rounds *= 2) {
-        size_t bytes = bits_at + 32;
-        bool more = false;
-        for (int k = 0; k < n; ++k) {
-            const vmc_batch_item &it = items[order[k]];
-            share[k] = ((it.walkers->W + rounds - 1) / rounds + 31) & ~31;
-            more = more || share[k] > 32;
-            bytes += row_bytes(it.lists->view) * (size_t)share[k];
-        }
-        if (bytes <= ctx->rates_bytes) break;
-        if (bytes - bits_at > kBitsCap && more) continue;
-        const cudaError_t e = grow_store(ctx, bytes);
-        if (e == cudaSuccess) break;
-        if (e != cudaErrorMemoryAllocation || !more) return cuda_check(ctx, e, "batched rate store");
+    if (step) {
+        plan.parts = ctx->batch_parts;
+        plan.rounds = ctx->batch_rounds;
+    } else {
+        vmc_status st = place_batch(ctx, n, items, order, plan);
+        if (st) return st;
     }
-    plan.rounds = rounds;
+    const int rounds = plan.rounds;
     const int n_tabs = rounds == 1 ? 1 : rounds + 1;
     std::string tab(sizeof(SysDesc) * n * n_tabs, '\0');
     SysDesc *d = (SysDesc *)&tab[0];
     int wb = 0, tb = 0;
-    size_t bit_off = bits_at;
     for (int k = 0; k < n; ++k) {
         const vmc_batch_item &it = items[order[k]];
+        const BatchPart &part = plan.parts[order[k]];
         plan.words = std::max(plan.words, it.lists->view.words);
-        d[k].bits = (uint32_t *)((char *)ctx->rates + bit_off);
-        bit_off += row_bytes(it.lists->view) * (size_t)share[k];
+        d[k].bits = (uint32_t *)((char *)ctx->rates + part.bits_at);
         d[k].w_first = 0;
         d[k].w_count = it.walkers->W;
         d[k].t_begin = tb;
@@ -1759,7 +1777,7 @@ static vmc_status prepare_batch(vmc_ctx *ctx, int n, const vmc_batch_item *items
         d[k].J = it.params->J;
         d[k].e_loc = it.d_e_loc;
         d[k].t_res = it.d_t_res;
-        d[k].rates = (u128 *)ctx->rates + rate_off[k];
+        d[k].rates = (u128 *)ctx->rates + part.rates_at;
         d[k].move_code = it.d_move_code;
         d[k].w_begin = wb;
         wb += it.walkers->W;
@@ -1769,9 +1787,10 @@ static vmc_status prepare_batch(vmc_ctx *ctx, int n, const vmc_batch_item *items
         int w = 0, t = 0;
         for (int k = 0; k < n; ++k) {
             SysDesc &x = d[(size_t)(r + 1) * n + k];
+            const int share = plan.parts[order[k]].share;
             x = d[k];
-            x.w_first = std::min(r * share[k], d[k].w_count);
-            x.w_count = std::min(share[k], d[k].w_count - x.w_first);
+            x.w_first = std::min(r * share, d[k].w_count);
+            x.w_count = std::min(share, d[k].w_count - x.w_first);
             x.w_begin = w;
             x.t_begin = t;
             w += x.w_count;
@@ -1803,15 +1822,19 @@ static vmc_status prepare_batch(vmc_ctx *ctx, int n, const vmc_batch_item *items
     return VMC_OK;
 }
 
-static std::string batch_signature(int n, const vmc_batch_item *items) {
-    std::string sig;
-    for (int k = 0; k < n; ++k) sig.append((const char *)&items[k].walkers->G, sizeof(void *));
-    return sig;
+// Are these the items whose rates the store holds (or fewer walkers of them)?
+static bool batch_stored(const vmc_ctx *ctx, int n, const vmc_batch_item *items) {
+    if (!items || ctx->batch_parts.empty() || (size_t)n != ctx->batch_parts.size()) return false;
+    for (int k = 0; k < n; ++k) {
+        const BatchPart &p = ctx->batch_parts[k];
+        if (!items[k].lists || p.G != items[k].walkers->G || items[k].walkers->W > p.W || !same_lists(p, items[k].lists)) return false;
+    }
+    return true;
 }
 
 vmc_status launch_local_energy_batch(vmc_ctx *ctx, int n, const vmc_batch_item *items) {
     BatchPlan plan;
-    vmc_status st = prepare_batch(ctx, n, items, plan);
+    vmc_status st = prepare_batch(ctx, n, items, false, plan);
     if (st) return st;
     const size_t se = plan.smem_eloc;
     if (!plan.fits) return set_err(ctx, VMC_ERR_ARG, "walker G table does not fit in shared memory");
@@ -1832,15 +1855,16 @@ vmc_status launch_local_energy_batch(vmc_ctx *ctx, int n, const vmc_batch_item *
         if (e == cudaSuccess) e = cudaGetLastError();
     }
     if (e != cudaSuccess) return cuda_check(ctx, e, "k_local_energy_batched");
-    ctx->rates_batch = batch_signature(n, items);
+    ctx->batch_parts = plan.parts;
+    ctx->batch_rounds = plan.rounds;
     return VMC_OK;
 }
 
 vmc_status launch_ctmc_step_batch(vmc_ctx *ctx, int n, const vmc_batch_item *items, uint64_t seed) {
-    if (ctx->rates_batch.empty() || ctx->rates_batch != batch_signature(n, items))
+    if (!batch_stored(ctx, n, items))
         return set_err(ctx, VMC_ERR_ARG, "vmc_local_energy_batch must precede vmc_ctmc_step_batch on the same items");
     BatchPlan plan;
-    vmc_status st = prepare_batch(ctx, n, items, plan);
+    vmc_status st = prepare_batch(ctx, n, items, true, plan);
     if (st) return st;
     const int total = plan.total, prec = plan.precision;
     const size_t sa = plan.smem_apply;
@@ -1860,7 +1884,7 @@ vmc_status launch_ctmc_step_batch(vmc_ctx *ctx, int n, const vmc_batch_item *ite
     }
     ctx->launches += 2;
     if (e == cudaSuccess) e = cudaGetLastError();
-    ctx->rates_batch.clear();
+    ctx->batch_parts.clear();
     return cuda_check(ctx, e, "k_ctmc_*_batched");
 }
 

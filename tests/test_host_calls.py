@@ -112,3 +112,46 @@ def test_batched_moves_need_their_own_energies(runtime, ctx, between):
     vmc.vmc_ctmc_step_batch(ctx, items, 3)
     for s in two:
         s.close()
+
+
+def _store_bytes(runtime, call):
+    a = runtime.counts()["live"]
+    call()
+    return runtime.counts()["live"] - a
+
+
+@pytest.mark.parametrize("later", [0, None])
+def test_batched_moves_keep_the_rate_store(runtime, ctx, later):
+    """Too little memory for every walker's rows: the energies run in rounds, and the moves read the store as it is,
+    whether or not there is more memory by then."""
+    two = _two(ctx)
+    items = fake_cudart.batch(two)
+    full = _store_bytes(runtime, lambda: vmc.vmc_local_energy_batch(ctx, items))
+    c2 = vmc.vmc_create(0, 0)
+    runtime.launches()
+    runtime.limit(full * 3 // 4)
+    vmc.vmc_local_energy_batch(c2, items)
+    assert sum("k_local_energy" in x for x in runtime.launches()) == 2
+    runtime.limit(later)
+    before = runtime.counts()
+    vmc.vmc_ctmc_step_batch(c2, items, 3)
+    assert runtime.counts() == before
+    assert sum("k_ctmc" in x for x in runtime.launches()) == 2
+    vmc.vmc_destroy(c2)
+    for s in two:
+        s.close()
+
+
+def test_moves_refuse_other_batch_items(runtime, ctx):
+    two = _two(ctx)
+    other = fake_cudart.System(ctx, S.named_system("H6"), 1, 1e-2)
+    vmc.vmc_local_energy_batch(ctx, fake_cudart.batch(two))
+    two[0].walkers.W += 1
+    assert "must precede" in _refused(vmc.vmc_ctmc_step_batch, ctx, fake_cudart.batch(two), 3)
+    two[0].walkers.W -= 1
+    keep, two[1].lists = two[1].lists, other.lists
+    assert "must precede" in _refused(vmc.vmc_ctmc_step_batch, ctx, fake_cudart.batch(two), 3)
+    two[1].lists = keep
+    vmc.vmc_ctmc_step_batch(ctx, fake_cudart.batch(two), 3)
+    for s in (*two, other):
+        s.close()
