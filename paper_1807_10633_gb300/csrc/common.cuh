@@ -48,6 +48,7 @@ struct vmc_ctx {
     // survives the gradient's use of ws
     void *rates = nullptr;
     size_t rates_bytes = 0;
+    size_t rates_refused = SIZE_MAX;   // the smallest store that could not be allocated
     void *bits = nullptr;        // in rates: the free-entry rows of the last vmc_local_energy's walkers
     int bits_whole = 0;          // they hold every walker of the last vmc_local_energy
     // rate store bookkeeping (vmc_local_energy -> vmc_ctmc_step)

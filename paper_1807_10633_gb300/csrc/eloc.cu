@@ -1548,8 +1548,10 @@ static cudaError_t eloc_batched_launch(const vmc_ctx *ctx, int nsm, size_t se, c
 }
 
 // Rate store and, behind it in the same allocation, the free-entry rows of one launch's walkers: at most
-// kBitsCap bytes of rows (but at least one tile of 32 walkers); a larger call runs in several launches of *chunk
-// walkers.  row = 0: no rows.  When the memory cannot be had the chunk is halved down to one tile.
+// kBitsCap bytes of rows (but those of 32 walkers at least); a larger call runs in several launches of *chunk
+// walkers.  row = 0: no rows.  When the memory cannot be had the chunk is halved, down to 32 walkers.  A size that
+// could not be had is not asked for again where fewer rows will do: the calls after the first find the store as it
+// is, allocate nothing and wait for nothing (they may be captured).
 constexpr size_t kBitsCap = (size_t)1 << 30;
 
 static size_t row_bytes(const ListsView &L) { return std::max<size_t>(32, sizeof(uint32_t) * (size_t)L.words); }
@@ -1566,9 +1568,16 @@ static cudaError_t grow_store(vmc_ctx *ctx, size_t bytes) {
         ctx->rates_bytes = 0;
     }
     const cudaError_t e = cudaMalloc(&ctx->rates, bytes);
-    if (e == cudaSuccess) ctx->rates_bytes = bytes;
-    else ctx->rates = nullptr;
-    if (e == cudaErrorMemoryAllocation) cudaGetLastError();
+    if (e == cudaSuccess) {
+        ctx->rates_bytes = bytes;
+        if (bytes >= ctx->rates_refused) ctx->rates_refused = SIZE_MAX;
+    } else {
+        ctx->rates = nullptr;
+    }
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        ctx->rates_refused = std::min(ctx->rates_refused, bytes);
+    }
     return e;
 }
 
@@ -1581,8 +1590,9 @@ static vmc_status ensure_store(vmc_ctx *ctx, size_t rates_bytes, size_t row, int
     }
     for (;; n = std::max(32, (n / 2 + 31) & ~31)) {
         const size_t bytes = r + row * (size_t)n + 32;     // a read of two words may run past the last row
-        cudaError_t e = cudaSuccess;
-        if (bytes > ctx->rates_bytes) e = grow_store(ctx, bytes);
+        if (bytes <= ctx->rates_bytes) break;
+        if (row && n > 32 && bytes >= ctx->rates_refused) continue;
+        const cudaError_t e = grow_store(ctx, bytes);
         if (e == cudaSuccess) break;
         if (e != cudaErrorMemoryAllocation || !row || n <= 32) return cuda_check(ctx, e, "rate store");
     }
@@ -1710,7 +1720,7 @@ static vmc_status place_batch(vmc_ctx *ctx, int n, const vmc_batch_item *items, 
         }
         const size_t bytes = at + 32;
         if (bytes <= ctx->rates_bytes) return VMC_OK;
-        if (bytes - bits_at > kBitsCap && more) continue;
+        if (more && (bytes - bits_at > kBitsCap || bytes >= ctx->rates_refused)) continue;
         const cudaError_t e = grow_store(ctx, bytes);
         if (e == cudaSuccess) return VMC_OK;
         if (e != cudaErrorMemoryAllocation || !more) return cuda_check(ctx, e, "batched rate store");

@@ -155,3 +155,32 @@ def test_moves_refuse_other_batch_items(runtime, ctx):
     vmc.vmc_ctmc_step_batch(ctx, fake_cudart.batch(two), 3)
     for s in (*two, other):
         s.close()
+
+
+@pytest.mark.parametrize("batched", [False, True])
+def test_short_memory_is_remembered(runtime, ctx, batched):
+    """Rows that did not fit are not asked for again: later calls allocate, free and wait for nothing, so that they can
+    be captured; rates that are needed are still asked for when there may be memory again."""
+    two = _two(ctx)
+    items = fake_cudart.batch(two)
+
+    def energy(c):
+        vmc.vmc_local_energy_batch(c, items) if batched else two[0].energy(ctx=c)
+    full = _store_bytes(runtime, lambda: energy(ctx))
+    big = fake_cudart.System(ctx, S.named_system("H6"), 100000, 1e-6)
+    c2 = vmc.vmc_create(0, 0)
+    runtime.limit(full * 3 // 4)
+    energy(c2)
+    before = runtime.counts()
+    runtime.limit(0, capturing=True)
+    energy(c2)
+    assert runtime.counts() == before
+    runtime.limit(0)
+    with pytest.raises(vmc.VmcError) as e:
+        big.energy(ctx=c2)
+    assert e.value.status == 3                           # VMC_ERR_OOM
+    runtime.limit()
+    big.energy(ctx=c2)
+    for s in (*two, big):
+        s.close()
+    vmc.vmc_destroy(c2)
