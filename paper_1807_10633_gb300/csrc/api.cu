@@ -13,6 +13,7 @@ vmc_status set_err(vmc_ctx *ctx, vmc_status st, const std::string &msg) {
 
 vmc_status cuda_check(vmc_ctx *ctx, cudaError_t e, const char *what) {
     if (e == cudaSuccess) return VMC_OK;
+    cudaGetLastError();      // reported here: the next call's launches are not blamed for it
     if (e == cudaErrorMemoryAllocation)
         return set_err(ctx, VMC_ERR_OOM, std::string(what) + ": " + cudaGetErrorString(e));
     return set_err(ctx, VMC_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));

@@ -38,7 +38,7 @@ cudaError_t launched(const void *f, dim3 g) {
 extern "C" {
 
 // ---- the tests' side
-void fake_set(uint64_t limit, int capturing) { st().limit = limit; st().capturing = capturing; st().last = cudaSuccess; }
+void fake_set(uint64_t limit, int capturing) { st().limit = limit; st().capturing = capturing; }
 void fake_counts(int64_t out[5]) {
     out[0] = st().mallocs; out[1] = st().frees; out[2] = st().uploads; out[3] = st().waits; out[4] = (int64_t)st().live;
 }

@@ -184,3 +184,16 @@ def test_short_memory_is_remembered(runtime, ctx, batched):
     for s in (*two, big):
         s.close()
     vmc.vmc_destroy(c2)
+
+
+def test_a_failed_allocation_is_reported_once(runtime, ctx):
+    """The runtime keeps an allocation's error until it is asked for: the call after it must not report it again."""
+    s = fake_cudart.System(ctx, S.named_system("H6"), 64, 1e-6)
+    out = [s._array(8 * k) for k in (144, 18, 18)]
+    runtime.limit(0)
+    with pytest.raises(vmc.VmcError) as e:
+        vmc.vmc_grad_logpsi(ctx, s.walkers, s.t, *out)
+    assert e.value.status == 3                           # VMC_ERR_OOM
+    vmc.vmc_log_psi(ctx, s.walkers, s.params, s.e)
+    runtime.limit()
+    s.close()
