@@ -1810,6 +1810,7 @@ static vmc_status prepare_batch(vmc_ctx *ctx, int n, const vmc_batch_item *items
         plan.tiles.push_back(t);
     }
     if (tab != ctx->batch_host) {
+        ctx->batch_host.clear();               // (until the new table is there)
         if (tab.size() > ctx->batch_desc_bytes) {
             if (ctx->batch_desc) { cudaStreamSynchronize(ctx->stream); cudaFree(ctx->batch_desc); }
             cudaError_t e = cudaMalloc(&ctx->batch_desc, tab.size());

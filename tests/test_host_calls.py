@@ -197,3 +197,29 @@ def test_a_failed_allocation_is_reported_once(runtime, ctx):
     vmc.vmc_log_psi(ctx, s.walkers, s.params, s.e)
     runtime.limit()
     s.close()
+
+
+
+def test_batch_table_that_could_not_grow(runtime, ctx):
+    """A failed allocation of the batch's table leaves none: the next call uploads one or reports the same, it does not
+    launch on the table that was freed."""
+    two = _two(ctx)
+    big, small = fake_cudart.batch(two), fake_cudart.batch(two[:1])
+    vmc.vmc_local_energy_batch(ctx, big)
+    c2 = vmc.vmc_create(0, 0)
+    two[0].energy(ctx=c2)
+    two[0].walkers.W = 1                                 # (the store is large enough)
+    vmc.vmc_local_energy_batch(c2, small)
+    runtime.launches()
+    for items in (big, small):
+        runtime.limit(0)
+        with pytest.raises(vmc.VmcError) as e:
+            vmc.vmc_local_energy_batch(c2, items)
+        assert e.value.status == 3                       # VMC_ERR_OOM
+    assert runtime.launches() == []
+    runtime.limit()
+    vmc.vmc_local_energy_batch(c2, small)
+    assert len(runtime.launches()) == 2
+    vmc.vmc_destroy(c2)
+    for s in two:
+        s.close()
