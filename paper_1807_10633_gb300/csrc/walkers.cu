@@ -150,6 +150,13 @@ __device__ void refresh_orbitals(int w, int sg, int M, int na, int nb, const uin
                                  uint16_t *virt_list, uint16_t *pos_all, uint32_t *occ_bits, uint16_t *s_occ,
                                  uint16_t *s_virt, uint8_t *mark);
 
+// Multipliers a / d are a times the reciprocal of the pivot.  That is not a normal number for |d| >= 2^1022, and
+// infinite for most subnormal d: there a and d are scaled by this power of two first (1 elsewhere).
+__device__ __forceinline__ double pivot_scale(double d) {
+    const uint32_t e = (uint32_t)((unsigned long long)__double_as_longlong(d) >> 52) & 0x7FFu;
+    return e == 0u ? 0x1p200 : (e >= 2045u ? 0x1p-200 : 1.0);
+}
+
 // LU with partial pivoting of the n x n FP64 matrix B in shared memory (row stride ld) by the whole CTA:
 // P B = L U, rows left in place; returns the row list rl (rl[k] = the row that is pivot k; perm, with
 // perm[k] = k on entry, or perm2).  Look-ahead: while warps 1.. update columns k+2.. of step k, warp 0
@@ -179,7 +186,10 @@ __device__ __forceinline__ const int *lu_factor(double *B, int n, int ld, int *p
         const double d = B[rout[k] * ld + k];
         const bool zero = ((unsigned long long)__double_as_longlong(d) << 1) == 0ull;   // +-0
         if (zero && lane == 0) *sing = 1;
-        const double dinv = zero ? 1.0 : __drcp_rn(d);
+        const double sc = pivot_scale(d);
+        if (!zero && sc != 1.0)
+            for (int r = k + 1 + lane; r < n; r += 32) B[rout[r] * ld + k] *= sc;
+        const double dinv = zero ? 1.0 : __drcp_rn(d * sc);
         for (int r = k + 1 + lane; r < n; r += 32) B[rout[r] * ld + k] *= dinv;
     };
     if (n > 0 && warp == 0) pivot(0, perm, perm2);
@@ -949,7 +959,13 @@ k_log_psi_warp(int W, int M, int na, int nb, const double *__restrict__ Ca, cons
                 zero = zero || z;
                 if (lane == k) dk = d;
                 if (lane == p) used = true;
-                const double f = used ? 0.0 : a[k] * (z ? 1.0 : __drcp_rn(d));
+                double f = used ? 0.0 : a[k], e = z ? 1.0 : d;
+                const double sc = pivot_scale(e);
+                if (sc != 1.0) {
+                    f *= sc;
+                    e *= sc;
+                }
+                f *= __drcp_rn(e);
 #pragma unroll
                 for (int c = k + 1; c < NP; ++c)
                     if (c < n) {
