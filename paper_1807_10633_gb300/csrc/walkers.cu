@@ -162,26 +162,27 @@ __device__ __forceinline__ double pivot_scale(double d) {
 // perm[k] = k on entry, or perm2).  Look-ahead: while warps 1.. update columns k+2.. of step k, warp 0
 // updates column k+1, picks the pivot of step k+1 into the other row list and scales its
 // multipliers, so the serial pivot work overlaps the FP64 update.  A zero pivot sets *sing.  Ends with a barrier.
-__device__ __forceinline__ const int *lu_factor(double *B, int n, int ld, int *perm, int *perm2, int *sing) {
+template <typename idx>
+__device__ __forceinline__ const idx *lu_factor(double *B, int n, int ld, idx *perm, idx *perm2, int *sing) {
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
-    auto pivot = [&](int k, const int *rin, int *rout) {      // warp 0 only
+    auto pivot = [&](int k, const idx *rin, idx *rout) {      // warp 0 only
         for (int r = lane; r < n; r += 32) rout[r] = rin[r];
         __syncwarp();
         // partial pivoting on |B[r][k]|, compared as the integer bits of |v| plus one (0: NaN or no
         // row), so the warp reductions run on the integer pipe; ties go to the lowest row
         unsigned long long best = 0ull;
-        int idx = k;
+        int at = k;
         for (int r = k + lane; r < n; r += 32) {
             const unsigned long long a =
                 (unsigned long long)__double_as_longlong(B[rout[r] * ld + k]) & 0x7FFFFFFFFFFFFFFFull;
             const unsigned long long key = a > 0x7FF0000000000000ull ? 0ull : a + 1ull;
-            if (key > best) { best = key; idx = r; }
+            if (key > best) { best = key; at = r; }
         }
         const uint32_t bh = (uint32_t)(best >> 32), bl = (uint32_t)best;
         const uint32_t mh = __reduce_max_sync(0xffffffffu, bh);
         const uint32_t ml = __reduce_max_sync(0xffffffffu, bh == mh ? bl : 0u);
-        idx = __reduce_min_sync(0xffffffffu, (bh == mh && bl == ml) ? idx : 0x7FFFFFFF);
-        if (lane == 0 && idx != k) { const int t = rout[k]; rout[k] = rout[idx]; rout[idx] = t; }
+        at = __reduce_min_sync(0xffffffffu, (bh == mh && bl == ml) ? at : 0x7FFFFFFF);
+        if (lane == 0 && at != k) { const idx t = rout[k]; rout[k] = rout[at]; rout[at] = t; }
         __syncwarp();
         const double d = B[rout[k] * ld + k];
         const bool zero = ((unsigned long long)__double_as_longlong(d) << 1) == 0ull;   // +-0
@@ -194,7 +195,7 @@ __device__ __forceinline__ const int *lu_factor(double *B, int n, int ld, int *p
     };
     if (n > 0 && warp == 0) pivot(0, perm, perm2);
     __syncthreads();
-    int *cur = perm2, *nxt = perm;
+    idx *cur = perm2, *nxt = perm;
     for (int k = 0; k + 1 < n; ++k) {
         const double *rowk = B + cur[k] * ld;
         if (warp == 0) {
@@ -220,7 +221,7 @@ __device__ __forceinline__ const int *lu_factor(double *B, int n, int ld, int *p
             }
         }
         __syncthreads();
-        int *t = cur; cur = nxt; nxt = t;
+        idx *t = cur; cur = nxt; nxt = t;
     }
     return cur;
 }
@@ -865,7 +866,8 @@ k_init_sums(ListsView L, int na, int nb, const real *__restrict__ Jsym, const ui
 
 // ln C[n] = sum_{p<q} J_pq n_p n_q + sum_p J_pp n_p over occupied spin orbitals s_so[0 .. ne): this thread's
 // terms t, t + stride, ...
-__device__ __forceinline__ double jastrow_terms(const double *__restrict__ J, int N2, const int *s_so, int ne, int t, int stride) {
+template <typename idx>
+__device__ __forceinline__ double jastrow_terms(const double *__restrict__ J, int N2, const idx *s_so, int ne, int t, int stride) {
     double part = 0.0;
     for (; t < ne * ne; t += stride) {
         const int x = t / ne, y = t - x * ne;
@@ -874,18 +876,19 @@ __device__ __forceinline__ double jastrow_terms(const double *__restrict__ J, in
     return part;
 }
 
-// ln|psi|, n_sigma > 32: one CTA per walker, each spin's determinant by the LU in shared memory.
+// ln|psi|, n_sigma > 32: one CTA per walker, each spin's determinant by the LU in shared memory (n_sigma up to 169: its
+// FP64 rows leave 2,600 bytes, so the lists hold 16-bit entries).
 __global__ void __launch_bounds__(VMC_THREADS)
 k_log_psi(int M, int na, int nb, const double *__restrict__ Ca, const double *__restrict__ Cb,
           const double *__restrict__ J, const uint16_t *occ_list, double *out, unsigned *status) {
     const int w = blockIdx.x, ne = na + nb, N2 = 2 * M;
     const int tid = threadIdx.x, nt = blockDim.x;
     extern __shared__ double sm[];
-    __shared__ int s_so[2 * VMC_MAX_M], perm[VMC_MAX_M], perm2[VMC_MAX_M];
+    __shared__ uint16_t s_so[2 * VMC_MAX_M], perm[VMC_MAX_M], perm2[VMC_MAX_M];
     __shared__ int s_sing;
     __shared__ double red[VMC_WARPS];
     const uint16_t *occ = occ_list + (size_t)w * ne;
-    for (int c = tid; c < ne; c += nt) s_so[c] = (c < na ? 0 : M) + occ[c];
+    for (int c = tid; c < ne; c += nt) s_so[c] = (uint16_t)((c < na ? 0 : M) + occ[c]);
     if (tid == 0) s_sing = 0;
     __syncthreads();
     double part = jastrow_terms(J, N2, s_so, ne, tid, nt);
@@ -898,9 +901,9 @@ k_log_psi(int M, int na, int nb, const double *__restrict__ Ca, const double *__
             const int r = t / n, x = t - r * n;
             sm[r * ld + x] = C[(size_t)occ[(sg ? na : 0) + r] * n + x];
         }
-        for (int k = tid; k < n; k += nt) perm[k] = k;
+        for (int k = tid; k < n; k += nt) perm[k] = (uint16_t)k;
         __syncthreads();
-        const int *rl = lu_factor(sm, n, ld, perm, perm2, &s_sing);
+        const uint16_t *rl = lu_factor(sm, n, ld, perm, perm2, &s_sing);
         for (int k = tid; k < n; k += nt) part += log(fabs(sm[rl[k] * ld + k]));
     }
     part = warp_sum_f64(part);

@@ -1,4 +1,5 @@
-"""ln|psi| (Sec. III.A) at the ends of its range: pivots whose reciprocals are no normal numbers (needs a GB300).
+"""ln|psi| (Sec. III.A) at the ends of its range: pivots whose reciprocals are no normal numbers, and the largest
+determinant that an SM's shared memory holds (needs a GB300).
 
 Reference: slogdet in FP64 of the occupied rows, the scaled column taken back to order one exactly (powers of two;
 the subnormal elements are rounded before, in both).  Tolerance of LU with partial pivoting as in
@@ -25,9 +26,10 @@ def _log_psi(M, na, nb, W, Ca, Cb, J, occ):
 
 
 # n on both sides of 16 and 32 (a warp's rows in registers, a CTA's in shared memory); pivots of a scaled first
-# column near 2^-1030 (subnormal) and 2^1022
+# column near 2^-1030 (subnormal) and 2^1022; n = 169, where rows and lists fill the shared memory
 @pytest.mark.parametrize("M,na,nb,W,ex", [(12, 5, 4, 5, -1030), (40, 20, 17, 3, -1030), (80, 40, 33, 3, -1030),
-                                          (12, 5, 4, 5, 1021), (80, 40, 20, 3, 1021), (40, 20, 32, 2, 0)])
+                                          (12, 5, 4, 5, 1021), (80, 40, 20, 3, 1021), (40, 20, 32, 2, 0),
+                                          (172, 169, 33, 2, 0)])
 def test_range(M, na, nb, W, ex):
     rng = np.random.default_rng(M + na)
     Ca, Cb = rng.uniform(0.6, 1.9, (M, na)) * rng.choice((-1.0, 1.0), (M, na)), rng.normal(size=(M, nb))
