@@ -363,7 +363,21 @@ static void build_flat(const ListsView &v, const HostLists &H, FlatLists &F) {
     align(256, 0);
 }
 
-// Effective list lengths for eps_run (host binary searches): the unit table and the alive bits.
+// Sets bits [b, e).
+static void fill_bits(std::vector<uint32_t> &bits, uint32_t b, uint32_t e) {
+    if (b == e) return;
+    const uint32_t first = ~0u << (b & 31u), last = ~0u >> (31u - ((e - 1) & 31u)), wb = b >> 5, we = (e - 1) >> 5;
+    if (wb == we) {
+        bits[wb] |= first & last;
+        return;
+    }
+    bits[wb] |= first;
+    std::fill(bits.begin() + wb + 1, bits.begin() + we, ~0u);
+    bits[we] |= last;
+}
+
+// Effective list lengths for eps_run (host binary searches): the unit table and the alive bits.  Word by word: a
+// change of eps_run costs the units and words, not the entries.
 vmc_status lists_set_eps(vmc_ctx *ctx, vmc_lists *L, double eps_run) {
     if (L->eps_run == eps_run) return VMC_OK;
     const ListsView &v = L->view;
@@ -379,7 +393,7 @@ vmc_status lists_set_eps(vmc_ctx *ctx, vmc_lists *L, double eps_run) {
             const uint32_t base = L->h_base[(size_t)g * 32 + lane];
             tab[(size_t)g * 32 + lane] = make_uint4((uint32_t)u.p | ((uint32_t)(u.kind == 0 ? 0 : u.q) << 16), base, n,
                                                     (uint32_t)(u.kind | (u.spin << 2)));
-            for (uint32_t e = base; e < base + n; ++e) alive[e >> 5] |= 1u << (e & 31u);
+            fill_bits(alive, base, base + n);
         }
     cudaError_t e;
     e = cudaMemcpyAsync((void *)v.unit_tab, tab.data(), sizeof(uint4) * tab.size(), cudaMemcpyHostToDevice, ctx->stream);
