@@ -312,21 +312,24 @@ struct FlatLists {
     std::vector<uint4> group;
 };
 
+// First the places of all units (serially: a few steps per unit), then the entries (in parallel: they are most of
+// the time, H60 at eps = 0 4.3 s for a build of 15 M entries appended one by one and 2.4 s so; 2.2 s before there were flat entries).
 static void build_flat(const ListsView &v, const HostLists &H, FlatLists &F) {
-    auto bits_d = [](uint32_t u) { double d = 0.0; uint64_t x = u; memcpy(&d, &x, 8); return d; };
-    auto bits_f = [](uint32_t u) { float f; memcpy(&f, &u, 4); return f; };
-    auto align = [&](size_t to, uint8_t cls) {     // fill up to a multiple of `to` entries
-        while (F.key.size() % to) {
-            if (F.key.size() % 32 == 0) F.wcls.push_back(cls);
-            F.key.push_back(0);
-            F.r32.push_back(make_float4(0.f, 0.f, 0.f, 0.f));
-            F.r64.push_back(make_double4_32a(0.0, 0.0, 0.0, 0.0));
-        }
+    size_t n = 0;                                  // entries so far
+    auto advance = [&](size_t k, uint8_t cls) {    // a word has the class of its first entry
+        n += k;
+        while (F.wcls.size() * 32 < n) F.wcls.push_back(cls);
+    };
+    auto align = [&](size_t to, uint8_t cls) { advance((to - n % to) % to, cls); };
+    auto list_of = [&](const UnitId &u, uint32_t &e0) {
+        const std::vector<uint32_t> &off = u.kind == 0 ? H.s_off : (u.kind == 1 ? H.ds_off : H.do_off);
+        e0 = off[u.list];
+        return off[u.list + 1] - e0;
     };
     F.base.assign((size_t)v.n_groups * 32, 0);
     for (int g = 0; g < v.n_groups; ++g) {
         align(64, 0);
-        uint4 info = make_uint4((uint32_t)(F.key.size() / 32), 0xFFFFFFFFu, 0, 0);
+        uint4 info = make_uint4((uint32_t)(n / 32), 0xFFFFFFFFu, 0, 0);
         int last = -1;
         for (int lane = 0; lane < 32; ++lane) {
             UnitId u;
@@ -340,27 +343,41 @@ static void build_flat(const ListsView &v, const HostLists &H, FlatLists &F) {
                          (uint32_t)((lane - u.q - u.p * ui) & 31) << 6;
             }
             if (u.kind == 2) info.w = (info.w & 0x7FFu) | (uint32_t)((lane - u.q) & 31) << 11;
-            if (u.kind == 2 && info.y == 0xFFFFFFFFu) info.y = (uint32_t)(F.key.size() / 32);
-            F.base[(size_t)g * 32 + lane] = (uint32_t)F.key.size();
-            const uint32_t *off = u.kind == 0 ? H.s_off.data() : (u.kind == 1 ? H.ds_off.data() : H.do_off.data());
-            for (uint32_t e = off[u.list]; e < off[u.list + 1]; ++e) {
-                const uint32_t ab = u.kind == 0 ? (uint32_t)H.s_a[e] | ((uint32_t)H.s_a[e] << 16)
-                                                : (u.kind == 1 ? H.ds_ab[e] : H.do_ab[e]);
-                const double x = u.kind == 0 ? 0.0 : (u.kind == 1 ? H.ds_v[e] : H.do_v[e]);
-                const uint32_t key = (ab & 0xFFu) | ((ab >> 16 & 0xFFu) << 8) | ((uint32_t)u.p << 16) | ((uint32_t)u.q << 24);
-                const uint32_t aux = u.kind == 0 ? (uint32_t)(u.spin * H.ns_pad) + e : 0u;
-                if (F.key.size() % 32 == 0) F.wcls.push_back(cls);
-                F.key.push_back(key);
-                F.r32.push_back(make_float4(bits_f(key), (float)x, 1.0f, bits_f(aux)));
-                F.r64.push_back(make_double4_32a(bits_d(key), x, 1.0, bits_d(aux)));
-            }
+            if (u.kind == 2 && info.y == 0xFFFFFFFFu) info.y = (uint32_t)(n / 32);
+            F.base[(size_t)g * 32 + lane] = (uint32_t)n;
+            uint32_t e0;
+            advance(list_of(u, e0), cls);
         }
         align(32, (uint8_t)std::max(0, last));
-        info.z = (uint32_t)(F.key.size() / 32);
+        info.z = (uint32_t)(n / 32);
         if (info.y == 0xFFFFFFFFu) info.y = info.z;
         F.group.push_back(info);
     }
     align(256, 0);
+    F.key.assign(n, 0);                            // unused places: key 0
+    F.r32.assign(n, make_float4(0.f, 0.f, 0.f, 0.f));
+    F.r64.assign(n, make_double4_32a(0.0, 0.0, 0.0, 0.0));
+    auto bits_d = [](uint32_t u) { double d = 0.0; uint64_t x = u; memcpy(&d, &x, 8); return d; };
+    auto bits_f = [](uint32_t u) { float f; memcpy(&f, &u, 4); return f; };
+#pragma omp parallel for schedule(dynamic, 32)
+    for (int t = 0; t < v.n_groups * 32; ++t) {
+        UnitId u;
+        if (!unit_of(v, t / 32, t % 32, u)) continue;
+        uint32_t e0;
+        const uint32_t len = list_of(u, e0);
+        for (uint32_t k = 0; k < len; ++k) {
+            const uint32_t e = e0 + k;
+            const size_t at = (size_t)F.base[t] + k;
+            const uint32_t ab = u.kind == 0 ? (uint32_t)H.s_a[e] | ((uint32_t)H.s_a[e] << 16)
+                                            : (u.kind == 1 ? H.ds_ab[e] : H.do_ab[e]);
+            const double x = u.kind == 0 ? 0.0 : (u.kind == 1 ? H.ds_v[e] : H.do_v[e]);
+            const uint32_t key = (ab & 0xFFu) | ((ab >> 16 & 0xFFu) << 8) | ((uint32_t)u.p << 16) | ((uint32_t)u.q << 24);
+            const uint32_t aux = u.kind == 0 ? (uint32_t)(u.spin * H.ns_pad) + e : 0u;
+            F.key[at] = key;
+            F.r32[at] = make_float4(bits_f(key), (float)x, 1.0f, bits_f(aux));
+            F.r64[at] = make_double4_32a(bits_d(key), x, 1.0, bits_d(aux));
+        }
+    }
 }
 
 // Sets bits [b, e).
