@@ -134,9 +134,7 @@ struct View {
     __device__ const real *Grow(int s, int slot) const {
         return s ? Gb + (size_t)slot * ldb : Ga + (size_t)slot * lda;
     }
-    const real *E;         // [2M] exp(S_p) for virtual p, 1/exp(S_p) for occupied p (nullptr: compute
-                           // from S on the fly)
-    const real *S;         // walker S in global (used when E == nullptr)
+    const real *S;         // walker S in global
     const real *F;         // walker F [2][ns_pad]
     CpsView C;             // correlator product (C.n_corr == 0: none)
     // its tables, staged in shared memory by the local energy (global otherwise): coefficient offsets,
@@ -149,9 +147,8 @@ struct View {
     __device__ int cur_of(int l) const { return cur ? cur[l] : voff[l] + (int)cidx[l]; }
     __device__ real coef(int k) const;
     __device__ real cinv_of(int l) const { return cinv ? cinv[l] : rrcp(coef(cur_of(l))); }
-    __device__ real Ev(int p) const { return E ? E[p] : rexp(S[p]); }              // p virtual
-    __device__ real Eiv(int p) const { return E ? E[p] : rrcp(rexp(S[p])); }       // p occupied
-    __device__ bool occ(int p) const { return !(pos[p] & 0x8000); }
+    __device__ real Ev(int p) const { return rexp(S[p]); }              // p virtual
+    __device__ real Eiv(int p) const { return rrcp(rexp(S[p])); }       // p occupied
 };
 
 // Correlator coefficient k in the table precision (the mixed form reads the FP32 copy).
@@ -1026,7 +1023,7 @@ __device__ __forceinline__ void select_walker(const ListsView &L, const WalkerAr
         const u128 Tl = T - before;   // threshold inside the group
         View<real> V;
         V.pos = A.pos + (size_t)w * N2; V.Ga = Gw; V.Gb = Gw + geo.g_off(1); V.lda = geo.na; V.ldb = geo.nb;
-        V.E = nullptr; V.S = Sw; V.F = (const real *)A.F + (size_t)w * 2 * L.ns_pad; V.geo = geo;
+        V.S = Sw; V.F = (const real *)A.F + (size_t)w * 2 * L.ns_pad; V.geo = geo;
         if (kC) cps_global(V, C, A.cps + (size_t)w * C.n_corr);
         const uint4 gi = __ldg(&L.group[gsel]);
         const bool single = gsel < (N2 + 31) / 32;
@@ -1135,7 +1132,7 @@ k_screened_moves(ListsView L, WalkerArgs A, CpsView C, int w_begin, int n_w, int
     const real *Gw = (const real *)A.G + (size_t)w * geo.g_stride;
     View<real> V;
     V.pos = A.pos + (size_t)w * N2; V.Ga = Gw; V.Gb = Gw + geo.g_off(1); V.lda = geo.na; V.ldb = geo.nb;
-    V.E = nullptr; V.S = (const real *)A.S + (size_t)w * N2; V.F = (const real *)A.F + (size_t)w * 2 * L.ns_pad;
+    V.S = (const real *)A.S + (size_t)w * N2; V.F = (const real *)A.F + (size_t)w * 2 * L.ns_pad;
     V.geo = geo;
     if (kC) cps_global(V, C, A.cps + (size_t)w * C.n_corr);
     const unsigned lt_mask = (1u << lane) - 1u;
@@ -1480,8 +1477,9 @@ static size_t eloc_smem_bytes(const ListsView &L, const vmc_walkers *Wk, const C
     return g + orb + own + warps + cps;
 }
 
-// Which walkers the local energy takes: G rows, exp(S), orbital map, 512 bytes per warp and the correlator
-// tables (site lists included) within 200 KB (the CTA's own sum stays within the 227 KB that it can have).
+// Which walkers the local energy takes: G rows, exp(S), orbital map, 512 bytes per warp and the correlator tables
+// within 200 KB.  The line counts the per-site correlator lists, which are no longer staged: what is refused stays
+// the same, and the CTA's own sum (eloc_smem_bytes) stays within the 227 KB that it can have.
 static bool eloc_fits(const vmc_walkers *Wk, const CpsView &C, int threads) {
     const size_t esz = Wk->precision == VMC_FP64 ? 8 : 4, M = (size_t)Wk->M, na = (size_t)Wk->n_alpha, nb = (size_t)Wk->n_beta;
     const size_t cps = C.n_corr ? esz * (size_t)((C.n_corr + 3) & ~3) + 4 * (2 * (size_t)C.n_corr + 1) + 4 * (M + 1) + 4 * (size_t)C.nnz : 0;

@@ -542,8 +542,9 @@ __device__ __forceinline__ double rcp_rn(double d) { return __drcp_rn(d); }
 __device__ __forceinline__ float rcp_rn(float d) { return __frcp_rn(d); }
 
 // kG: G from the CUDA cores at the end (otherwise on the tensor cores by another kernel; a build without that part
-// needs fewer registers: no spills at three CTAs per SM for n <= 80 in FP64, and six CTAs for n <= 32, whose steps are
-// latency: H61, 5,003 walkers, FP64: 1.10 -> 0.97 ms).
+// needs fewer registers: the FP64 kernel spills 76 bytes at three CTAs per SM for n <= 80, 8 at four for n <= 64 and
+// none at six for n <= 32, whose steps are latency: H61, 5,003 walkers, FP64: 1.10 -> 0.97 ms).  The bounds are those
+// of that build for both: with G the FP64 kernel for n <= 32 spills 584 bytes at six CTAs (other bounds not timed).
 template <typename real, int R, bool kG>
 __global__ void __launch_bounds__(kGJ * kGJ, sizeof(real) == 4 ? (R <= 5 ? 4 : 2) : (R <= 2 ? 6 : R <= 4 ? 4 : R <= 5 ? 3 : 1))
 k_refresh_gj(int M, int na, int nb, const real *__restrict__ Ca, const real *__restrict__ Cb,
@@ -738,7 +739,7 @@ __global__ void k_convert_c(int M, int na, int nb, const double *__restrict__ Ca
 }
 
 // Jastrow sums S_p, and (full init only) Fock sums and the diagonal energy.
-// Jastrow sums S_p = sum_{k occ, k != p} J_kp for a block of kSumWalkers walkers (thread = p): each
+// Jastrow sums S_p = sum_{k occ, k != p} J_kp for a block of kSumWalkers walkers (thread = two p): each
 // walker's occupied rows of the symmetric J copy are added in ascending order, one add per
 // occupied orbital (the rows are L2 resident).
 // (Full init only:) Fock sums F and the diagonal energy, one walker per block.
