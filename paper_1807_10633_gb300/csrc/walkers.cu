@@ -151,18 +151,22 @@ __device__ void refresh_orbitals(int w, int sg, int M, int na, int nb, const uin
                                  uint16_t *s_virt, uint8_t *mark);
 
 // Multipliers a / d are a times the reciprocal of the pivot.  That is not a normal number for |d| >= 2^1022, and
-// infinite for most subnormal d: there a and d are scaled by this power of two first (1 elsewhere).
-__device__ __forceinline__ double pivot_scale(double d) {
+// infinite for most subnormal d (and for 0, which callers set to 1): far_pivot, one test of the exponent.  ln|psi|
+// takes a and d times pivot_scale there.
+__device__ __forceinline__ bool far_pivot(double d) {
     const uint32_t e = (uint32_t)((unsigned long long)__double_as_longlong(d) >> 52) & 0x7FFu;
-    return e == 0u ? 0x1p200 : (e >= 2045u ? 0x1p-200 : 1.0);
+    return e - 1u >= 2044u;
 }
+__device__ __forceinline__ double pivot_scale(double d) { return fabs(d) < 1.0 ? 0x1p200 : 0x1p-200; }
 
 // LU with partial pivoting of the n x n FP64 matrix B in shared memory (row stride ld) by the whole CTA:
 // P B = L U, rows left in place; returns the row list rl (rl[k] = the row that is pivot k; perm, with
 // perm[k] = k on entry, or perm2).  Look-ahead: while warps 1.. update columns k+2.. of step k, warp 0
 // updates column k+1, picks the pivot of step k+1 into the other row list and scales its
 // multipliers, so the serial pivot work overlaps the FP64 update.  A zero pivot sets *sing.  Ends with a barrier.
-template <typename idx>
+// kScale: pivots whose reciprocal is no normal number are scaled (not in the recompute, whose FP32 tables could not
+// hold the inverse: one more product on the serial pivot path took H160, 32,768 walkers, from 33.6 to 36.5 ms).
+template <bool kScale, typename idx>
 __device__ __forceinline__ const idx *lu_factor(double *B, int n, int ld, idx *perm, idx *perm2, int *sing) {
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
     auto pivot = [&](int k, const idx *rin, idx *rout) {      // warp 0 only
@@ -187,10 +191,11 @@ __device__ __forceinline__ const idx *lu_factor(double *B, int n, int ld, idx *p
         const double d = B[rout[k] * ld + k];
         const bool zero = ((unsigned long long)__double_as_longlong(d) << 1) == 0ull;   // +-0
         if (zero && lane == 0) *sing = 1;
-        const double sc = pivot_scale(d);
-        if (!zero && sc != 1.0)
-            for (int r = k + 1 + lane; r < n; r += 32) B[rout[r] * ld + k] *= sc;
-        const double dinv = zero ? 1.0 : __drcp_rn(d * sc);
+        double dinv = zero ? 1.0 : __drcp_rn(d);
+        if (kScale && far_pivot(d) && !zero) {
+            for (int r = k + 1 + lane; r < n; r += 32) B[rout[r] * ld + k] *= pivot_scale(d);
+            dinv = __drcp_rn(d * pivot_scale(d));
+        }
         for (int r = k + 1 + lane; r < n; r += 32) B[rout[r] * ld + k] *= dinv;
     };
     if (n > 0 && warp == 0) pivot(0, perm, perm2);
@@ -260,7 +265,7 @@ k_init_tables_mixed(int M, int na, int nb, const double *__restrict__ Ca, const 
     }
     __syncthreads();
     __shared__ int perm2[VMC_MAX_M];
-    const int *rl = lu_factor(B, n, ld, perm, perm2, &s_sing);
+    const int *rl = lu_factor<false>(B, n, ld, perm, perm2, &s_sing);
     if (s_sing && tid == 0) atomicOr(status, VMC_DEV_SINGULAR);
     // reciprocals of U's diagonal (one FP64 division per row, not per element; n <= 128)
     __shared__ double rdiag[VMC_MAX_M / 2];
@@ -904,7 +909,7 @@ k_log_psi(int M, int na, int nb, const double *__restrict__ Ca, const double *__
         }
         for (int k = tid; k < n; k += nt) perm[k] = (uint16_t)k;
         __syncthreads();
-        const uint16_t *rl = lu_factor(sm, n, ld, perm, perm2, &s_sing);
+        const uint16_t *rl = lu_factor<true>(sm, n, ld, perm, perm2, &s_sing);
         for (int k = tid; k < n; k += nt) part += log(fabs(sm[rl[k] * ld + k]));
     }
     part = warp_sum_f64(part);
@@ -959,15 +964,14 @@ k_log_psi_warp(int W, int M, int na, int nb, const double *__restrict__ Ca, cons
                 const uint32_t ml = __reduce_max_sync(0xffffffffu, kh == mh ? kl : 0u);
                 const int p = __ffs(__ballot_sync(0xffffffffu, kh == mh && kl == ml && !used)) - 1;
                 const double d = __shfl_sync(0xffffffffu, a[k], p);
-                const bool z = ((unsigned long long)__double_as_longlong(d) << 1) == 0ull;      // +-0
-                zero = zero || z;
                 if (lane == k) dk = d;
                 if (lane == p) used = true;
-                double f = used ? 0.0 : a[k], e = z ? 1.0 : d;
-                const double sc = pivot_scale(e);
-                if (sc != 1.0) {
-                    f *= sc;
-                    e *= sc;
+                double f = used ? 0.0 : a[k], e = d;
+                if (far_pivot(d)) {
+                    const bool z = ((unsigned long long)__double_as_longlong(d) << 1) == 0ull;  // +-0
+                    zero = zero || z;
+                    f *= z ? 1.0 : pivot_scale(d);
+                    e = z ? 1.0 : d * pivot_scale(d);
                 }
                 f *= __drcp_rn(e);
 #pragma unroll
