@@ -53,7 +53,11 @@ typedef struct vmc_ctx vmc_ctx;       /* device, stream, workspace, status word 
 typedef struct vmc_lists vmc_lists;   /* device-resident screened integral lists */
 
 /* Create a context on CUDA device `device`; `cuda_stream` is a cudaStream_t (NULL = legacy
-   default stream).  The context allocates a small status word and grows a workspace on demand. */
+   default stream).  The context allocates a small status word, and on demand, kept until vmc_destroy:
+   a workspace (gradient partial sums) and the rate store of the local energy, which holds every
+   walker's rates (24 bytes per group, vmc_lists_layout) and the free-entry bits of as many walkers as
+   one launch takes (a bit per list entry and walker; at most 1 GiB, less if that cannot be had:
+   more walkers then run in several launches). */
 vmc_status vmc_create(vmc_ctx **ctx, int device, void *cuda_stream);
 vmc_status vmc_destroy(vmc_ctx *ctx);
 /* Replace the stream used by later calls (cudaStream_t). */
