@@ -312,8 +312,9 @@ struct FlatLists {
     std::vector<uint4> group;
 };
 
-// First the places of all units (serially: a few steps per unit), then the entries (in parallel: they are most of
-// the time, H60 at eps = 0 4.3 s for a build of 15 M entries appended one by one and 2.4 s so; 2.2 s before there were flat entries).
+// First the places of all units (serially: a few steps per unit), then the entries.  From a million on they are
+// written in parallel (H60 at eps = 0, 15 M: a build of 2.4 s, 4.3 s with the entries appended one by one, 2.2 s before
+// there were flat entries); below, the threads of one more region can cost a short build milliseconds on a busy host.
 static void build_flat(const ListsView &v, const HostLists &H, FlatLists &F) {
     size_t n = 0;                                  // entries so far
     auto advance = [&](size_t k, uint8_t cls) {    // a word has the class of its first entry
@@ -359,7 +360,7 @@ static void build_flat(const ListsView &v, const HostLists &H, FlatLists &F) {
     F.r64.assign(n, make_double4_32a(0.0, 0.0, 0.0, 0.0));
     auto bits_d = [](uint32_t u) { double d = 0.0; uint64_t x = u; memcpy(&d, &x, 8); return d; };
     auto bits_f = [](uint32_t u) { float f; memcpy(&f, &u, 4); return f; };
-#pragma omp parallel for schedule(dynamic, 32)
+#pragma omp parallel for schedule(dynamic, 32) if (n >= (size_t)1 << 20)
     for (int t = 0; t < v.n_groups * 32; ++t) {
         UnitId u;
         if (!unit_of(v, t / 32, t % 32, u)) continue;

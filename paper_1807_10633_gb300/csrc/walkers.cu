@@ -927,7 +927,7 @@ k_log_psi(int M, int na, int nb, const double *__restrict__ Ca, const double *__
 // unused row with the largest |a_k| (keys compared as integers; NaN lowest, ties to the lowest row) is
 // broadcast element by element and eliminated from the other unused rows.  At these sizes the CTA-wide
 // elimination is barriers and latency: 4,096 walkers of H40 took 952 us with it (one FP64 division and an
-// integer division per updated element), 244 us with this kernel.  By count, not by profile: a warp-wide FP64
+// integer division per updated element), 221 us with this kernel.  By count, not by profile: a warp-wide FP64
 // instruction takes 16 clocks of an SM's FP64 pipe whatever lanes are active, so the n^2 / 2 row updates come to
 // about 80 us and the n reciprocals to a like amount.
 constexpr int kLogWarps = 8;     // four walkers per CTA
