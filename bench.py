@@ -156,8 +156,8 @@ class Clocks:
 # warp instructions (smsp__inst_executed.sum), from the capture summarised in
 # profiles/k_local_energy_mixed_h160_w4096.md.  They describe the kernel source with this digest
 # only; any later change of the kernel's file reports traffic as null until it is captured again.
-ELOC_COUNTERS = {"sha256": "60394967b2157dd5532e1a73589eb86585ed0fcf87f153270902cfbbe68aab2c",
-                 "system": "H160", "eps": 1e-6, "dram_bytes_per_walker": 119893.3, "l2_bytes_per_walker": 759253.3,
+ELOC_COUNTERS = {"sha256": "380534b3b876cd5568b7554784d02b53809bfa0d744b175170ba011042ac3c6f",
+                 "system": "H160", "eps": 1e-6, "dram_bytes_per_walker": 119938.0, "l2_bytes_per_walker": 759263.5,
                  "warp_inst_per_walker": 173000.4}
 
 
